@@ -184,6 +184,8 @@ int collapse(dds_ctx *ctx) {
   return DDS_OK;
 }
 
+}  // namespace
+
 // Mirror x_a -> -x_a maps the segment of (t, b) onto itself and b onto +-b.
 bool mirror_ok(const double *t, const double *b, int a) {
   const int a1 = (a + 1) % 3, a2 = (a + 2) % 3;
@@ -199,8 +201,6 @@ int mirror_parity(const double *b, int a, int c) {
   const int qi = I[c] == a ? -1 : 1, qj = J[c] == a ? -1 : 1;
   return -sb * qi * qj;
 }
-
-}  // namespace
 
 size_t zfour_symmetry(const double *field_t, const double *field_b, int fe, Shape *sh) {
   ZSym &zs = sh->zs;

@@ -13,8 +13,13 @@
 // The table of G over all offsets is wrapped into the zero-padded periodic grid
 // (offset D -> index D mod P), transformed by an FP64 R2C FFT, and because the
 // table is odd (G(-D) = -G(D)) its spectrum is purely imaginary: only Im / (Px Py Pz)
-// is kept, in FP32, laid out per tile of the fused z pass.
+// is kept, in FP32, laid out per tile of the fused z pass.  Oddness, and the mirrors a
+// field has, also halve the table and each transform (see below).
 #include <math.h>
+
+#include <algorithm>
+#include <utility>
+#include <vector>
 
 #include <cuda_fp16.h>
 
@@ -29,102 +34,120 @@ struct V3 {
   double x, y, z;
 };
 __host__ __device__ __forceinline__ V3 v3(double x, double y, double z) { return V3{x, y, z}; }
-__device__ __forceinline__ V3 operator+(V3 a, V3 b) { return v3(a.x + b.x, a.y + b.y, a.z + b.z); }
-__device__ __forceinline__ V3 operator-(V3 a, V3 b) { return v3(a.x - b.x, a.y - b.y, a.z - b.z); }
-__device__ __forceinline__ V3 operator*(double s, V3 a) { return v3(s * a.x, s * a.y, s * a.z); }
-__device__ __forceinline__ double dot(V3 a, V3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
-__device__ __forceinline__ V3 cross(V3 a, V3 b) {
+__host__ __device__ __forceinline__ V3 operator+(V3 a, V3 b) { return v3(a.x + b.x, a.y + b.y, a.z + b.z); }
+__host__ __device__ __forceinline__ V3 operator*(double s, V3 a) { return v3(s * a.x, s * a.y, s * a.z); }
+__host__ __device__ __forceinline__ double dot(V3 a, V3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
+__host__ __device__ __forceinline__ V3 cross(V3 a, V3 b) {
   return v3(a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x);
 }
 __device__ __forceinline__ double comp(V3 a, int i) { return i == 0 ? a.x : (i == 1 ? a.y : a.z); }
 
-// Bracket of Eq. 6 at one segment end, divided by R_t^2.  R joins the observer and
-// the end point (either orientation, see segment_stress).  S in xx,yy,zz,xy,xz,yz.
-__device__ void eq6_end(V3 R, V3 t, V3 b, double k1, double S[6]) {
-  const double Rn = sqrt(dot(R, R));
-  const double L = dot(R, t);
-  const V3 Rt = R + Rn * t;
-  const double iRt2 = 1.0 / dot(Rt, Rt);
-  const V3 rho = R - L * t;
-  const V3 u = cross(b, Rt);          // enters [b R_t t]^sym
-  const V3 w = cross(b, t);           // enters [b t R_t]^sym
-  const double k2 = 0.5 * k1 * dot(u, t);   // (b, R_t, t) / (2 (1 - nu))
-  const double LR = L / Rn;
-  const int ia[6] = {0, 1, 2, 0, 0, 1};
-  const int ic[6] = {0, 1, 2, 1, 2, 2};
-#pragma unroll
-  for (int q = 0; q < 6; ++q) {
-    const int a = ia[q], c = ic[q];
-    const double ta = comp(t, a), tc = comp(t, c);
-    const double Ra = comp(Rt, a), Rc = comp(Rt, c);
-    const double s1 = 0.5 * (comp(u, a) * tc + comp(u, c) * ta);
-    const double s2 = 0.5 * (comp(w, a) * Rc + comp(w, c) * Ra);
-    const double phi = 2.0 * iRt2 * (comp(rho, a) * Rc + comp(rho, c) * Ra + LR * Ra * Rc);
-    const double dl = (a == c) ? 1.0 : 0.0;
-    S[q] = iRt2 * (s1 - k1 * s2 - k2 * (dl + ta * tc + phi));
-  }
-}
+// A box (cell or subcell) as a source: half its chord along t, and mu / pi times its
+// volume over the chord.
+struct Box {
+  double hl, f;
+};
 
-// Stress (Pa) of the segment from -hl t to +hl t at observer r (relative to the
-// segment centre), Burgers vector b.  Zero for the observer at the centre.
-__device__ void segment_stress(V3 r, double hl, V3 t, V3 b, double mu, double nu, double out[6]) {
-  if (r.x == 0.0 && r.y == 0.0 && r.z == 0.0) {
-#pragma unroll
-    for (int q = 0; q < 6; ++q) out[q] = 0.0;
-    return;
-  }
-  V3 RA = (-hl) * t - r;   // observer -> A
-  V3 RB = hl * t - r;      // observer -> B
-  const double cA = dot(RA, t) / sqrt(dot(RA, RA));
-  const double cB = dot(RB, t) / sqrt(dot(RB, RB));
-  if (cA + cB < 0.0) {     // observer ahead of the segment: use the other form of Eq. 6
-    RA = (-1.0) * RA;
-    RB = (-1.0) * RB;
-  }
-  const double k1 = 1.0 / (1.0 - nu);
-  double SA[6], SB[6];
-  eq6_end(RA, t, b, k1, SA);
-  eq6_end(RB, t, b, k1, SB);
-  const double pref = mu * 0.31830988618379067154;   // mu / pi
-#pragma unroll
-  for (int q = 0; q < 6; ++q) out[q] = pref * (SB[q] - SA[q]);
-}
+// NF fields of one line direction: what their coefficients share.
+template <int NF> struct Fields {
+  V3 t;
+  V3 b[NF], w[NF];          // Burgers vectors, b x t
+  double k1;                // 1 / (1 - nu)
+  Box cell, sub;
+};
 
-__device__ __forceinline__ double box_chord(const double hb[3], V3 t) {
-  double dl = 1e300;
-  const double tt[3] = {t.x, t.y, t.z};
+// Adds weight * (box coefficient) of every field at observer offset r (from the box
+// centre) to acc[f][xx, yy, zz, xy, xz, yz].
+//
+// Eq. 6 at the ends A, B = -+hl t, with R from the observer to the end, splits into the
+// part of R across the line, which both ends share, and the one along it:
+//   R = rho + L t,  R_t = R + |R| t = rho + q t,  q = L + |R|,  R_t^2 = 2 |R| q,
+// so the bracket of Eq. 6 is a sum of tensors in (rho, t, b) common to both ends, each
+// times a scalar of the end.  With g = 1 / (2 |R|), i = g / q = 1 / R_t^2, l = L / |R|:
+//   S = i (V - k1 X) + g (1 - k1) W
+//       - k1 beta [ i (1 + t t) / 2 + i^2 (2 + l) rho rho + 2 g^3 (rho t + t rho) + l g^2 t t ],
+// V = sym(b x rho, t), W = sym(w, t), X = sym(w, rho), w = b x t, beta = (b x rho) . t;
+// only the differences of the five scalars between B and A remain per field.  Two
+// reciprocal square roots and one division serve all fields of the direction: FP64
+// units are scarce (1/64 of the FP32 rate), and this is about a tenth of the operations
+// of evaluating Eq. 6 per end and field (GaN layer, five fields: tables 234 -> 12.4 ms
+// with the offsets the symmetries leave; 15 replica shells on 64x64x8, two fields: 374 ->
+// 15.4 ms).  The observer at the centre gives 0.
+template <int NF>
+__device__ __forceinline__ void box_add(const Fields<NF> &F, V3 r, const Box &box, double weight, double (&acc)[NF][6]) {
+  if (r.x == 0.0 && r.y == 0.0 && r.z == 0.0) return;
+  const double rt = dot(r, F.t);
+  V3 rho = v3(rt * F.t.x - r.x, rt * F.t.y - r.y, rt * F.t.z - r.z);
+  const double rho2 = dot(rho, rho);
+  double LA = -box.hl - rt, LB = box.hl - rt;
+  const double RA2 = LA * LA + rho2, RB2 = LB * LB + rho2;
+  const double rsA = rsqrt(RA2), rsB = rsqrt(RB2);
+  double lA = LA * rsA, lB = LB * rsB;
+  if (lA + lB < 0.0) {     // observer ahead of the segment: R from the end to the observer
+    LA = -LA;
+    LB = -LB;
+    lA = -lA;
+    lB = -lB;
+    rho = (-1.0) * rho;
+  }
+  // q = L + |R|; beside the segment (L < 0) the same as rho^2 / (|R| - L)
+  double qA = fabs(LA) + RA2 * rsA, qB = fabs(LB) + RB2 * rsB;
+  if (LA < 0.0) qA = rho2 / qA;
+  if (LB < 0.0) qB = rho2 / qB;
+  const double iq = 1.0 / (qA * qB);
+  const double gA = 0.5 * rsA, gB = 0.5 * rsB;
+  const double iA = gA * (iq * qB), iB = gB * (iq * qA);
+  const double ga2 = gA * gA, gb2 = gB * gB;
+  const double s = weight * box.f;
+  const double d0 = s * (iB - iA), d1 = s * (gB - gA);
+  const double d2 = s * (iB * iB * (2.0 + lB) - iA * iA * (2.0 + lA));
+  const double d3 = 2.0 * s * (gb2 * gB - ga2 * gA);
+  const double d4 = s * (lB * gb2 - lA * ga2);
+  const double h0 = 0.5 * d0, dt = h0 + d4;
+  constexpr int IA[6] = {0, 1, 2, 0, 0, 1}, IC[6] = {0, 1, 2, 1, 2, 2};
+  double T[6];             // the tensor of the beta term, shared by the fields
+  const V3 p = d2 * rho + d3 * F.t, z = d3 * rho + dt * F.t;     // rho (d2 rho + d3 t) + t (d3 rho + dt t)
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    if (tt[a] != 0.0) dl = fmin(dl, hb[a] / fabs(tt[a]));
-  return dl;
-}
-
-// g(r) for a box of edges hb: (V / dl) sigma^AB(r).
-__device__ void box_coef(V3 r, const double hb[3], V3 t, V3 b, double mu, double nu, double out[6]) {
-  const double dl = box_chord(hb, t);
-  const double vol = hb[0] * hb[1] * hb[2];
-  segment_stress(r, 0.5 * dl, t, b, mu, nu, out);
-  const double f = vol / dl;
+  for (int c = 0; c < 6; ++c)
+    T[c] = (IA[c] == IC[c] ? h0 : 0.0) + comp(rho, IA[c]) * comp(p, IC[c]) + comp(F.t, IA[c]) * comp(z, IC[c]);
 #pragma unroll
-  for (int q = 0; q < 6; ++q) out[q] *= f;
+  for (int f = 0; f < NF; ++f) {
+    const V3 w = F.w[f];
+    const double kb = F.k1 * dot(w, rho);                // -k1 beta
+    // d0 (V - k1 X) + d1 (1 - k1) W = sym(t, d0 v + d1 (1 - k1) w) - sym(w, d0 k1 rho), halves folded in
+    const V3 x = h0 * cross(F.b[f], rho) + (0.5 * d1 * (1.0 - F.k1)) * w;
+    const V3 y = (-h0 * F.k1) * rho;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      const int a = IA[c], e = IC[c];
+      double v;
+      if (a == e) v = 2.0 * (comp(F.t, a) * comp(x, a) + comp(w, a) * comp(y, a));
+      else v = comp(F.t, a) * comp(x, e) + comp(F.t, e) * comp(x, a) + comp(w, a) * comp(y, e) + comp(w, e) * comp(y, a);
+      acc[f][c] += kb * T[c] + v;
+    }
+  }
 }
 
 __device__ __forceinline__ V3 offset_pos(const CoefGeom &g, int i, int j, int k) {
   return v3((double)i * g.h[0], (double)j * g.h[1], (double)k * g.h[2]);
 }
 
-// Near-field coefficient: the term of subcell difference index q of the
-// (2m-1)^3 lattice, times its multiplicity.
-__device__ __forceinline__ double near_term(const CoefGeom &g, V3 base, int q, V3 t, V3 b,
-                                            double out[6]) {
+__device__ __forceinline__ int near_terms(const CoefGeom &g) {
+  return (2 * g.m[0] - 1) * (2 * g.m[1] - 1) * (2 * g.m[2] - 1);
+}
+
+// Near-field coefficient: adds the term of subcell difference index q of the (2m-1)^3
+// lattice, times its multiplicity over the number of subcells.
+template <int NF>
+__device__ __forceinline__ void near_add(const CoefGeom &g, const Fields<NF> &F, V3 base, int q, double weight,
+                                         double (&acc)[NF][6]) {
   const int Dx = 2 * g.m[0] - 1, Dy = 2 * g.m[1] - 1;
   const int dx = q % Dx - (g.m[0] - 1);
   const int dy = (q / Dx) % Dy - (g.m[1] - 1);
   const int dz = q / (Dx * Dy) - (g.m[2] - 1);
   const double mult = (double)((g.m[0] - abs(dx)) * (g.m[1] - abs(dy)) * (g.m[2] - abs(dz)));
   const V3 r = base + v3(dx * g.hs[0], dy * g.hs[1], dz * g.hs[2]);
-  box_coef(r, g.hs, t, b, g.mu, g.nu, out);
-  return mult;
+  box_add<NF>(F, r, F.sub, weight * mult / (double)(g.m[0] * g.m[1] * g.m[2]), acc);
 }
 
 // Near field: |(i dx, j dy, k dz)|^2 < rn2, as ((x*x + y*y) + z*z) in round-to-nearest
@@ -132,40 +155,6 @@ __device__ __forceinline__ double near_term(const CoefGeom &g, V3 base, int q, V
 __device__ __forceinline__ bool near_dev(const CoefGeom &g, int i, int j, int k) {
   const double x = __dmul_rn((double)i, g.h[0]), y = __dmul_rn((double)j, g.h[1]), z = __dmul_rn((double)k, g.h[2]);
   return __dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)) < g.rn2;
-}
-
-// Coefficient of one source cell at cell offset (i, j, k): subdivided near the target
-// (mean over target subcells of the sum over source subcells), one segment otherwise.
-__device__ void coef_cell(const CoefGeom &g, int i, int j, int k, V3 t, V3 b, double out[6]) {
-  const V3 base = offset_pos(g, i, j, k);
-  if (!near_dev(g, i, j, k)) {
-    box_coef(base, g.h, t, b, g.mu, g.nu, out);
-    return;
-  }
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  const int D = (2 * g.m[0] - 1) * (2 * g.m[1] - 1) * (2 * g.m[2] - 1);
-  for (int d = 0; d < D; ++d) {
-    double s[6];
-    const double mult = near_term(g, base, d, t, b, s);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) acc[c] += mult * s[c];
-  }
-  const double iM = 1.0 / (double)(g.m[0] * g.m[1] * g.m[2]);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) out[c] = acc[c] * iM;
-}
-
-// With periodic boundary conditions (Sec. 4, Eq. 13): the sum over the replicas of the
-// source cell, r_i + (k Lx, l Ly, 0), |k|, |l| <= n_shells.
-// Replica sum of Eq. 13 around in-plane offset (i, j): images (i + kk nx, j + ll ny).
-__device__ void coef_replicas(const CoefGeom &g, int i, int j, int k, V3 t, V3 b, double w, double acc[6]) {
-  for (int kk = -g.n_shells; kk <= g.n_shells; ++kk)
-    for (int ll = -g.n_shells; ll <= g.n_shells; ++ll) {
-      double s[6];
-      coef_cell(g, i + kk * g.nx, j + ll * g.ny, k, t, b, s);
-#pragma unroll
-      for (int c = 0; c < 6; ++c) acc[c] += w * s[c];
-    }
 }
 
 // Minimal image of offset i for period n, in (-n/2, n/2]; at the tie n/2 (n even) also
@@ -182,105 +171,186 @@ __device__ __forceinline__ int min_images(int i, int n, int r[2], double w[2]) {
   return 2;
 }
 
-__device__ void coef_any(const CoefGeom &g, int i, int j, int k, V3 t, V3 b, double out[6]) {
-  if (g.n_shells <= 0) {
-    coef_cell(g, i, j, k, t, b, out);
-    return;
+// Share `lane` of S of the coefficient at cell offset (i, j, k): one segment, or near the
+// target the mean over target subcells of the sum over source subcells; with periodic
+// boundary conditions (Sec. 4, Eq. 13) the sum over the replicas of the source cell,
+// r_i + (k Lx, l Ly, 0), |k|, |l| <= n_shells, around the in-system offset or its minimal
+// images (ties averaged: odd and periodic).  The lanes take the images in turn, and the
+// subcell differences of every near image together (one near image is up to a few
+// hundred terms), so they finish at about the same time.  Every lane of a warp calls
+// this with the same number of images; `lanes`: the warp's mask of this offset's lanes.
+template <int NF, int S>
+__device__ __forceinline__ void coef_share(const CoefGeom &g, const Fields<NF> &F, int i, int j, int k, int lane,
+                                           unsigned lanes, double (&acc)[NF][6]) {
+  const int n = g.n_shells, side = 2 * n + 1, images = side * side;
+  int rx[2] = {i, 0}, ry[2] = {j, 0};
+  double wx[2] = {1.0, 0.0}, wy[2] = {1.0, 0.0};
+  int nxr = 1, nyr = 1;
+  if (n > 0 && g.periodic) {
+    nxr = min_images(i, g.nx, rx, wx);
+    nyr = min_images(j, g.ny, ry, wy);
   }
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  if (!g.periodic) {
-    coef_replicas(g, i, j, k, t, b, 1.0, acc);
-  } else {             // shells centred on the minimal image, ties averaged (odd, periodic)
-    int rx[2], ry[2];
-    double wx[2], wy[2];
-    const int nxr = min_images(i, g.nx, rx, wx), nyr = min_images(j, g.ny, ry, wy);
-    for (int a = 0; a < nxr; ++a)
-      for (int c2 = 0; c2 < nyr; ++c2) coef_replicas(g, rx[a], ry[c2], k, t, b, wx[a] * wy[c2], acc);
-  }
-#pragma unroll
-  for (int c = 0; c < 6; ++c) out[c] = acc[c];
+  const int terms = near_terms(g);
+  for (int a = 0; a < nxr; ++a)
+    for (int b = 0; b < nyr; ++b) {
+      const double wt = wx[a] * wy[b];
+      for (int m0 = 0; m0 < images; m0 += S) {
+        const int m = m0 + lane;
+        const int ii = rx[a] + (m / side - n) * g.nx, jj = ry[b] + (m % side - n) * g.ny;
+        const bool near = m < images && near_dev(g, ii, jj, k);
+        if (m < images && !near) box_add<NF>(F, offset_pos(g, ii, jj, k), F.cell, wt, acc);
+        unsigned mask = S > 1 ? __ballot_sync(lanes, near) & lanes : (near ? 1u : 0u);
+        while (mask) {                        // this offset's near images, all its lanes on each
+          const int bit = __ffs(mask) - 1;
+          mask &= mask - 1;
+          const int q = m0 + (S > 1 ? bit % S : 0);
+          const V3 base = offset_pos(g, rx[a] + (q / side - n) * g.nx, ry[b] + (q % side - n) * g.ny, k);
+          for (int d = lane; d < terms; d += S) near_add<NF>(g, F, base, d, wt, acc);
+        }
+      }
+    }
 }
 
 // ---- coefficients at listed offsets (parity queries) ------------------------
-__global__ void k_table_at(CoefGeom g, V3 t, V3 b, long n, const int *ijk, double *out) {
+__global__ void k_table_at(CoefGeom g, Fields<1> F, long n, const int *ijk, double *out) {
   const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (q >= n) return;
-  double acc[6];
-  coef_any(g, ijk[3 * q], ijk[3 * q + 1], ijk[3 * q + 2], t, b, acc);
+  double acc[1][6] = {{0, 0, 0, 0, 0, 0}};
+  coef_share<1, 1>(g, F, ijk[3 * q], ijk[3 * q + 1], ijk[3 * q + 2], 0, 0u, acc);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) out[6 * q + c] = acc[c];
+  for (int c = 0; c < 6; ++c) out[6 * q + c] = acc[0][c];
 }
 
-// ---- padded table: far formula everywhere, gaps zero -------------------------
-// tab[c][kz][ky][kx], kx < px.  Offset D maps to index D mod P; indices with no
-// offset of magnitude < n (the padding gap) hold 0.
-__global__ void k_table_far(CoefGeom g, V3 t, V3 b, int nx, int ny, int nz, int px, int py, int pz,
-                            double *tab) {
-  const long P = (long)px * py * pz;
-  const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (idx >= P) return;
-  const int ix = (int)(idx % px), iy = (int)((idx / px) % py), iz = (int)(idx / ((long)px * py));
-  const int i = ix < nx ? ix : ix - px;
-  const int j = iy < ny ? iy : iy - py;
-  const int k = iz < nz ? iz : iz - pz;
-  double s[6] = {0, 0, 0, 0, 0, 0};
-  if (i > -nx && j > -ny && k > -nz) {
-    if (g.n_shells > 0) coef_any(g, i, j, k, t, b, s);     // replica sums include the near field
-    else box_coef(offset_pos(g, i, j, k), g.h, t, b, g.mu, g.nu, s);
-  }
+// ---- coefficient table of the fields of one line direction --------------------
+// Only offsets no symmetry gives: k >= 0 (the table is odd, G(-D) = -G(D)); i >= 0 when
+// every field has the x mirror, j >= 0 when every field has the y mirror.  Row r of an
+// axis with n cells holds offset r, or r - (2n - 1) from r = n on.
+struct Tab {
+  int nx, ny, nz;           // grid
+  int mx, my;               // mirrors used
+  int rx, ry;               // rows stored along x and y
+};
+__host__ __device__ __forceinline__ long tab_size(const Tab &T) { return (long)T.nz * T.ry * T.rx; }
+
+// One segment per offset (near offsets are overwritten by k_table_near).
+template <int NF>
+__global__ void __launch_bounds__(256) k_table_far(CoefGeom g, Fields<NF> F, Tab T, double *tab) {
+  const long N = tab_size(T), idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (idx >= N) return;
+  const int ir = (int)(idx % T.rx), jr = (int)((idx / T.rx) % T.ry), k = (int)(idx / ((long)T.rx * T.ry));
+  const int i = ir < T.nx ? ir : ir - (2 * T.nx - 1), j = jr < T.ny ? jr : jr - (2 * T.ny - 1);
+  double acc[NF][6] = {};
+  box_add<NF>(F, offset_pos(g, i, j, k), F.cell, 1.0, acc);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) tab[c * P + idx] = s[c];
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) tab[(f * 6 + c) * N + idx] = acc[f][c];
 }
 
-// One block per near offset: reduce the subcell-difference lattice and overwrite.
-__global__ void k_table_near(CoefGeom g, V3 t, V3 b, int px, int py, int pz, const int *ijk,
-                             double *tab) {
+// Replica sums: S lanes per offset.
+template <int NF, int S>
+__global__ void __launch_bounds__(256) k_table_pbc(CoefGeom g, Fields<NF> F, Tab T, double *tab) {
+  const long N = tab_size(T), idx = (blockIdx.x * (long)blockDim.x + threadIdx.x) / S;
+  if (idx >= N) return;                       // all lanes of an offset together
+  const int lane = threadIdx.x % S;
+  const unsigned lanes = S == 32 ? 0xffffffffu : ((1u << S) - 1u) << ((threadIdx.x & 31) / S * S);
+  const int ir = (int)(idx % T.rx), jr = (int)((idx / T.rx) % T.ry), k = (int)(idx / ((long)T.rx * T.ry));
+  const int i = ir < T.nx ? ir : ir - (2 * T.nx - 1), j = jr < T.ny ? jr : jr - (2 * T.ny - 1);
+  double acc[NF][6] = {};
+  coef_share<NF, S>(g, F, i, j, k, lane, lanes, acc);
+#pragma unroll
+  for (int f = 0; f < NF; ++f)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      double v = acc[f][c];
+      for (int o = S / 2; o > 0; o >>= 1) v += __shfl_xor_sync(lanes, v, o);
+      if (lane == 0) tab[(f * 6 + c) * N + idx] = v;
+    }
+}
+
+// One block per near offset (rows of the table): reduce the subcell-difference lattice.
+template <int NF>
+__global__ void __launch_bounds__(128) k_table_near(CoefGeom g, Fields<NF> F, Tab T, const int *ijk, double *tab) {
   const int q = blockIdx.x;
   const int i = ijk[3 * q], j = ijk[3 * q + 1], k = ijk[3 * q + 2];
   const V3 base = offset_pos(g, i, j, k);
-  const int D = (2 * g.m[0] - 1) * (2 * g.m[1] - 1) * (2 * g.m[2] - 1);
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int d = threadIdx.x; d < D; d += blockDim.x) {
-    double s[6];
-    const double mult = near_term(g, base, d, t, b, s);
+  double acc[NF][6] = {};
+  const int terms = near_terms(g);
+  for (int d = threadIdx.x; d < terms; d += blockDim.x) near_add<NF>(g, F, base, d, 1.0, acc);
+  __shared__ double red[4][NF * 6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) acc[c] += mult * s[c];
-  }
-  __shared__ double red[32][6];
+  for (int f = 0; f < NF; ++f)
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    double v = acc[c];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][c] = v;
-  }
+    for (int c = 0; c < 6; ++c) {
+      double v = acc[f][c];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][f * 6 + c] = v;
+    }
   __syncthreads();
-  if (threadIdx.x < 6) {
+  if (threadIdx.x < NF * 6) {
     double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w][threadIdx.x];
-    const long P = (long)px * py * pz;
-    const int ix = i >= 0 ? i : i + px, iy = j >= 0 ? j : j + py, iz = k >= 0 ? k : k + pz;
-    const long idx = ((long)iz * py + iy) * px + ix;
-    tab[threadIdx.x * P + idx] = v / (double)(g.m[0] * g.m[1] * g.m[2]);
+    for (int w = 0; w < 4; ++w) v += red[w][threadIdx.x];
+    const int ir = i >= 0 ? i : i + 2 * T.nx - 1, jr = j >= 0 ? j : j + 2 * T.ny - 1;
+    tab[threadIdx.x * tab_size(T) + ((long)k * T.ry + jr) * T.rx + ir] = v;
   }
 }
 
-// ---- FP64 FFT of the padded table -----------------------------------------
-// R2C along x: lines of 2M reals -> M+1 complex (row pitch M+1).
+// ---- FP64 FFT of the table ---------------------------------------------------
+// The table of (component, field) wrapped into the padded grid is real and odd, so its
+// transform is imaginary, and only half of each transform is work:
+//   x: real-to-complex lines of 2M points, layers k >= 0 only;
+//   y: layers k >= 0 only.  With the x mirror the x spectra are real or imaginary (one
+//      number per bin): two columns form one complex column, rows ky <= py/2 remain, and
+//      an x-even and an x-odd component share one real line (their sum: its spectrum's
+//      real part belongs to the even one, the imaginary part to the odd one);
+//   z: h(-z) = -conj h(z) gives the layers k < 0; two columns h1 + i h2 are transformed
+//      as one, whose spectrum is i S1 - S2.
+// FP64 arithmetic bounds every pass.  Full transforms of every padded value took 7.3 ms
+// per component of the GaN layer (256x256x128, padded 512x512x256: 2.3 x, 3.4 y, 1.6 z);
+// with the symmetries 2.0 ms (0.65 x, 0.93 y, 0.46 z).
+
+// Components of one launch: line set s transforms component ce[s], plus the x-odd one
+// co[s] when >= 0, into the spectra of slots se[s] and so[s]; sx, sy: mirror parities.
+struct Comps {
+  int sets, slots;
+  int ce[6], co[6], se[6], so[6];
+  int sx[6], sy[6];         // by component
+  int comp_of[6];           // by slot
+  int off;                  // first component of the field in the table (6 f)
+};
+
+// x: W lines (rows of the table) per block.  Without the x mirror: out[slot][k][jr][M + 1]
+// complex; with it one number per bin: the real part (x-even component), or the imaginary
+// part (x-odd).
 template <int M>
-__global__ void __launch_bounds__(128) k_r2c_lines_d(const double *in, long nlines, double2 *out,
-                                                     const double2 *tw) {
+__global__ void __launch_bounds__(128) k_x_lines_d(Tab T, Comps C, const double *tab, double *out, const double2 *tw) {
   constexpr int W = 4, LD = W + 1, NT = 128;
   extern __shared__ double2 sm_d[];
   double2 *buf = sm_d;
-  const long l0 = (long)blockIdx.x * W;
-  const int tid = threadIdx.x;
+  const long lines = (long)T.nz * T.ry, l0 = (long)blockIdx.x * W;
+  const int tid = threadIdx.x, set = blockIdx.y;
+  const int ce = C.ce[set], co = C.co[set];
+  const long N = tab_size(T);
+  const double *te = tab + (C.off + ce) * N, *to = co >= 0 ? tab + (C.off + co) * N : nullptr;
+  const double pe = C.sx[ce], po = co >= 0 ? C.sx[co] : 0.0;
+  auto value = [&](long line, int n) {        // sample n of the wrapped line
+    const int i = n < T.nx ? n : n - 2 * M;
+    if (i <= -T.nx) return 0.0;
+    const long row = line * T.rx;
+    if (!T.mx) return __ldg(te + row + (i >= 0 ? i : i + 2 * T.nx - 1));
+    const int a = abs(i);
+    double v = __ldg(te + row + a);
+    if (i < 0) v *= pe;
+    if (to != nullptr) {
+      const double u = __ldg(to + row + a);
+      v += i < 0 ? po * u : u;
+    }
+    return v;
+  };
   for (int e = tid; e < W * M; e += NT) {
     const int w = e / M, n = e % M;
     double2 z = make_double2(0.0, 0.0);
-    if (l0 + w < nlines) {
-      const double *src = in + (l0 + w) * (2L * M) + 2 * n;
-      z = make_double2(src[0], src[1]);
-    }
+    if (l0 + w < lines) z = make_double2(value(l0 + w, 2 * n), value(l0 + w, 2 * n + 1));
     buf[n * LD + w] = z;
   }
   __syncthreads();
@@ -288,41 +358,126 @@ __global__ void __launch_bounds__(128) k_r2c_lines_d(const double *in, long nlin
   const double2 *tw2 = tw + tw_offset(2 * M);
   for (int e = tid; e < W * (M + 1); e += NT) {
     const int w = e / (M + 1), k = e % (M + 1);
-    if (l0 + w >= nlines) continue;
+    if (l0 + w >= lines) continue;
     const double2 a = buf[(k % M) * LD + w];
     const double2 c = buf[((M - k) % M) * LD + w];
-    // E = (Z[k] + conj Z[M-k]) / 2,  O = (Z[k] - conj Z[M-k]) / 2i,  X = E + W^k O
-    const double2 E = make_double2(0.5 * (a.x + c.x), 0.5 * (a.y - c.y));
-    const double2 O = make_double2(0.5 * (a.y + c.y), -0.5 * (a.x - c.x));
+    // 2 E = Z[k] + conj Z[M-k],  2 O = (Z[k] - conj Z[M-k]) / i,  X = E + W^k O
+    const double2 E = make_double2(a.x + c.x, a.y - c.y);
+    const double2 O = make_double2(a.y + c.y, c.x - a.x);
     const double2 wk = (k < M) ? tw2[k] : make_double2(-1.0, 0.0);
-    const double2 X = make_double2(E.x + wk.x * O.x - wk.y * O.y, E.y + wk.x * O.y + wk.y * O.x);
-    out[(l0 + w) * (M + 1) + k] = X;
+    const long o = (l0 + w) * (M + 1) + k, S = lines * (M + 1);
+    if (!T.mx) {
+      reinterpret_cast<double2 *>(out)[C.se[set] * S + o] =
+          make_double2(0.5 * (E.x + wk.x * O.x - wk.y * O.y), 0.5 * (E.y + wk.x * O.y + wk.y * O.x));
+    } else {
+      if (pe > 0.0 || to != nullptr) out[C.se[set] * S + o] = 0.5 * (E.x + wk.x * O.x - wk.y * O.y);
+      else out[C.se[set] * S + o] = 0.5 * (E.y + wk.x * O.y + wk.y * O.x);
+      if (to != nullptr) out[C.so[set] * S + o] = 0.5 * (E.y + wk.x * O.y + wk.y * O.x);
+    }
   }
 }
 
-// C2C along a strided axis: element n of column c of batch o at
-// data[o * os + n * rs + c], c < ncols; tiles of W adjacent columns.
-template <int P, int W>
-__global__ void __launch_bounds__(256) k_cols_d(double2 *data, long os, long rs, long ncols,
-                                                const double2 *tw) {
-  constexpr int LD = W, NT = 256;
+// y: padded row iy of layer k is table row j = iy, or iy - py (zero in the gap).  Without
+// the x mirror W complex columns per tile, out[slot][k][ky < py][M + 1]; with it (PAIR) W
+// pairs of columns, out[slot][k][ky <= py/2][M + 1], multiplied by i for x-odd components.
+template <int P, int W, bool PAIR>
+__global__ void __launch_bounds__(256) k_y_cols_d(Tab T, Comps C, int M, const double *in, double2 *out, const double2 *tw) {
+  constexpr int NT = 256;
   extern __shared__ double2 sm_d[];
   double2 *buf = sm_d;
-  const long tiles = (ncols + W - 1) / W;
-  const long o = blockIdx.x / tiles;
-  const long c0 = (blockIdx.x % tiles) * W;
-  double2 *base = data + o * os + c0;
+  const int cols = M + 1, tiles = PAIR ? (cols + 2 * W - 1) / (2 * W) : (cols + W - 1) / W;
+  const int k = blockIdx.x / tiles, c0 = (blockIdx.x % tiles) * (PAIR ? 2 * W : W), slot = blockIdx.y;
+  const int comp = C.comp_of[slot];
   const int tid = threadIdx.x;
+  const long base = ((long)slot * T.nz + k) * T.ry;
   for (int e = tid; e < P * W; e += NT) {
     const int n = e / W, w = e % W;
-    buf[n * LD + w] = (c0 + w < ncols) ? base[n * rs + w] : make_double2(0.0, 0.0);
+    const int j = n < T.ny ? n : n - P;
+    double2 v = make_double2(0.0, 0.0);
+    if (j > -T.ny) {
+      const int jr = j >= 0 ? j : (T.my ? -j : j + 2 * T.ny - 1);
+      const double sg = j < 0 && T.my ? (double)C.sy[comp] : 1.0;
+      const long row = (base + jr) * cols;
+      if (PAIR) {
+        const int c = c0 + 2 * w;
+        if (c < cols) v.x = sg * __ldg(in + row + c);
+        if (c + 1 < cols) v.y = sg * __ldg(in + row + c + 1);
+      } else if (c0 + w < cols) {
+        v = __ldg(reinterpret_cast<const double2 *>(in) + row + c0 + w);
+        v.x *= sg;
+        v.y *= sg;
+      }
+    }
+    buf[n * W + w] = v;
   }
   __syncthreads();
-  fft_tile<P, W, LD, NT, false, false, false>(buf, tw + tw_offset(P), tid);
-  for (int e = tid; e < P * W; e += NT) {
-    const int n = e / W, w = e % W;
-    if (c0 + w < ncols) base[n * rs + w] = buf[n * LD + w];
+  fft_tile<P, W, W, NT, false, false, false>(buf, tw + tw_offset(P), tid);
+  if (!PAIR) {
+    double2 *dst = out + ((long)slot * T.nz + k) * P * cols;
+    for (int e = tid; e < P * W; e += NT) {
+      const int n = e / W, w = e % W;
+      if (c0 + w < cols) dst[(long)n * cols + c0 + w] = buf[n * W + w];
+    }
+  } else {
+    const bool odd = C.sx[comp] < 0;
+    double2 *dst = out + ((long)slot * T.nz + k) * (P / 2 + 1) * cols;
+    for (int e = tid; e < (P / 2 + 1) * 2 * W; e += NT) {
+      const int n = e / (2 * W), q = e % (2 * W), w = q / 2;
+      if (c0 + q >= cols) continue;
+      const double2 a = buf[n * W + w], b = buf[((P - n) % P) * W + w];
+      // columns f1 + i f2, both real: F1 = (C[k] + conj C[-k]) / 2, F2 = (C[k] - conj C[-k]) / 2i
+      double2 v = (q & 1) ? make_double2(0.5 * (a.y + b.y), 0.5 * (b.x - a.x))
+                          : make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
+      if (odd) v = make_double2(-v.y, v.x);
+      dst[(long)n * cols + c0 + q] = v;
+    }
   }
+}
+
+// z: pairs of adjacent columns of in[slot][k < nz][cols]; out[slot][kz < P][cols], the
+// imaginary part of the transform.
+template <int P, int W>
+__global__ void __launch_bounds__(256) k_z_cols_d(int nz, long cols, const double2 *in, double *out, const double2 *tw) {
+  constexpr int NT = 256;
+  extern __shared__ double2 sm_d[];
+  double2 *buf = sm_d;
+  const long c0 = (long)blockIdx.x * 2 * W;
+  const int slot = blockIdx.y, tid = threadIdx.x;
+  in += (long)slot * nz * cols;
+  out += (long)slot * P * cols;
+  for (int e = tid; e < (P / 2 + 1) * W; e += NT) {
+    const int n = e / W, w = e % W;
+    const long c = c0 + 2 * w;
+    double2 a = make_double2(0.0, 0.0), b = a;
+    if (n < nz && c < cols) a = __ldg(in + n * cols + c);
+    if (n < nz && c + 1 < cols) b = __ldg(in + n * cols + c + 1);
+    buf[n * W + w] = make_double2(a.x - b.y, a.y + b.x);                       // h1 + i h2
+    if (n > 0 && n < P / 2) buf[(P - n) * W + w] = make_double2(-a.x - b.y, a.y - b.x);   // -conj h1 - i conj h2
+  }
+  __syncthreads();
+  fft_tile<P, W, W, NT, false, false, false>(buf, tw + tw_offset(P), tid);
+  for (int e = tid; e < P * 2 * W; e += NT) {
+    const int n = e / (2 * W), q = e % (2 * W);
+    if (c0 + q >= cols) continue;
+    const double2 v = buf[n * W + q / 2];
+    out[n * cols + c0 + q] = (q & 1) ? -v.x : v.y;
+  }
+}
+
+// The imaginary part at (kx, ky, kz) of out[kz][ky][kx]; fold != 0: only ky <= py/2 are
+// held, and g(kx, -ky, -kz) = fold * g(kx, ky, kz) gives the others.
+__device__ __forceinline__ double spec_at(const double *spec, int M, int py, int pz, int fold, int kx, int ky, int kz) {
+  double s = 1.0;
+  int rows = py;
+  if (fold != 0) {
+    rows = py / 2 + 1;
+    if (ky > py / 2) {
+      ky = py - ky;
+      kz = kz == 0 ? 0 : pz - kz;
+      s = fold;
+    }
+  }
+  return s * spec[((long)kz * rows + ky) * (M + 1) + kx];
 }
 
 // Imaginary part of the spectrum of component c of field e, scaled, into the layout
@@ -337,10 +492,10 @@ __device__ __forceinline__ void store_val(__half *p, double v) { *p = __float2ha
 
 // Largest |Im| of one spectrum (for the FP16 scale); bit patterns of non-negative
 // doubles order like unsigned integers.
-__global__ void k_absmax_imag(const double2 *spec, long n, unsigned long long *out) {
+__global__ void k_absmax_imag(const double *spec, long n, unsigned long long *out) {
   double m = 0.0;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-    m = fmax(m, fabs(spec[i].y));
+    m = fmax(m, fabs(spec[i]));
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
@@ -352,7 +507,7 @@ __global__ void k_store_scale(const unsigned long long *amax, double scale, floa
 }
 
 template <typename OT>
-__global__ void k_extract(const double2 *spec, int M, int py, int pz, int wz, int zg, int fe, int e, int c,
+__global__ void k_extract(const double *spec, int fold, int M, int py, int pz, int wz, int zg, int fe, int e, int c,
                           double scale, const unsigned long long *amax, OT *kspec) {
   const int cw = zg > 0 ? 32 / zg : wz;                  // columns per tile
   const int E = zg > 0 ? pz / zg : 0;                     // registers per lane
@@ -383,7 +538,7 @@ __global__ void k_extract(const double2 *spec, int M, int py, int pz, int wz, in
     ky = (int)(tau - tiles_main) * cw + w;
     kx = M;
   }
-  double v = spec[((long)kz * py + ky) * (M + 1) + kx].y * scale;
+  double v = spec_at(spec, M, py, pz, fold, kx, ky, kz) * scale;
   if (amax != nullptr) {                 // FP16 storage: values relative to the largest
     const double m = __longlong_as_double((long long)*amax) * scale;
     if (m > 0.0) v /= m;
@@ -399,7 +554,7 @@ __global__ void k_extract(const double2 *spec, int M, int py, int pz, int wz, in
 // those with ky <= py/2 when every field has the x-mirror parity (ZSym::xall) -- then
 // the Nyquist tiles (kx = M).
 template <typename OT>
-__global__ void k_extract_four(const double2 *spec, Shape sh, int e, int c, double scale,
+__global__ void k_extract_four(const double *spec, int fold, Shape sh, int e, int c, double scale,
                                const unsigned long long *amax, OT *kspec) {
   constexpr int V = 16 / (int)sizeof(OT);
   const int W = sh.wz, R1 = sh.pz / 8, M = sh.M, py = sh.py, fe = sh.fe;
@@ -418,7 +573,7 @@ __global__ void k_extract_four(const double2 *spec, Shape sh, int e, int c, doub
     ky = (int)(s - main_tiles) * W + w;
     kx = M;
   }
-  double v = spec[((long)(k1 + R1 * k2) * py + ky) * (M + 1) + kx].y * scale;
+  double v = spec_at(spec, M, py, sh.pz, fold, kx, ky, k1 + R1 * k2) * scale;
   if (amax != nullptr) {                 // FP16 storage: values relative to the largest
     const double m = __longlong_as_double((long long)*amax) * scale;
     if (m > 0.0) v /= m;
@@ -427,52 +582,80 @@ __global__ void k_extract_four(const double2 *spec, Shape sh, int e, int c, doub
   store_val(&kspec[dst], v);
 }
 
+template <typename K>
+cudaError_t big_smem(K kernel, size_t smem) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
 template <int M>
-cudaError_t r2c_lines(const double *in, long nlines, double2 *out, const double2 *tw, cudaStream_t s) {
+cudaError_t x_lines(const Tab &T, const Comps &C, const double *tab, double *out, const double2 *tw, cudaStream_t s) {
   const size_t smem = sizeof(double2) * M * 5;
-  cudaError_t err = cudaFuncSetAttribute(k_r2c_lines_d<M>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+  cudaError_t err = big_smem(k_x_lines_d<M>, smem);
   if (err != cudaSuccess) return err;
-  k_r2c_lines_d<M><<<(unsigned)((nlines + 3) / 4), 128, smem, s>>>(in, nlines, out, tw);
+  const dim3 grid((unsigned)(((long)T.nz * T.ry + 3) / 4), C.sets);
+  k_x_lines_d<M><<<grid, 128, smem, s>>>(T, C, tab, out, tw);
   return cudaGetLastError();
 }
 
 template <int P>
-cudaError_t cols_fft(double2 *data, long nbatch, long os, long rs, long ncols, const double2 *tw,
-                     cudaStream_t s) {
+cudaError_t y_cols(const Tab &T, const Comps &C, int M, const double *in, double2 *out, const double2 *tw, cudaStream_t s) {
   constexpr int W = P >= 512 ? 4 : 8;
   const size_t smem = sizeof(double2) * P * W;
-  cudaError_t err = cudaFuncSetAttribute(k_cols_d<P, W>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+  cudaError_t err = T.mx ? big_smem(k_y_cols_d<P, W, true>, smem) : big_smem(k_y_cols_d<P, W, false>, smem);
   if (err != cudaSuccess) return err;
-  const long tiles = (ncols + W - 1) / W;
-  k_cols_d<P, W><<<(unsigned)(tiles * nbatch), 256, smem, s>>>(data, os, rs, ncols, tw);
+  const int per = T.mx ? 2 * W : W;
+  const dim3 grid((unsigned)((long)T.nz * ((M + per) / per)), C.slots);      // ceil((M + 1) / per) tiles per layer
+  if (T.mx) k_y_cols_d<P, W, true><<<grid, 256, smem, s>>>(T, C, M, in, out, tw);
+  else k_y_cols_d<P, W, false><<<grid, 256, smem, s>>>(T, C, M, in, out, tw);
   return cudaGetLastError();
 }
 
-cudaError_t r2c_dispatch(int M, const double *in, long nlines, double2 *out, const double2 *tw,
-                         cudaStream_t s) {
+template <int P>
+cudaError_t z_cols(int nz, long cols, int slots, const double2 *in, double *out, const double2 *tw, cudaStream_t s) {
+  constexpr int W = P >= 512 ? 4 : 8;
+  const size_t smem = sizeof(double2) * P * W;
+  cudaError_t err = big_smem(k_z_cols_d<P, W>, smem);
+  if (err != cudaSuccess) return err;
+  const dim3 grid((unsigned)((cols + 2 * W - 1) / (2 * W)), slots);
+  k_z_cols_d<P, W><<<grid, 256, smem, s>>>(nz, cols, in, out, tw);
+  return cudaGetLastError();
+}
+
+cudaError_t x_dispatch(int M, const Tab &T, const Comps &C, const double *tab, double *out, const double2 *tw,
+                       cudaStream_t s) {
   switch (M) {
-    case 16: return r2c_lines<16>(in, nlines, out, tw, s);
-    case 32: return r2c_lines<32>(in, nlines, out, tw, s);
-    case 64: return r2c_lines<64>(in, nlines, out, tw, s);
-    case 128: return r2c_lines<128>(in, nlines, out, tw, s);
-    case 256: return r2c_lines<256>(in, nlines, out, tw, s);
-    case 512: return r2c_lines<512>(in, nlines, out, tw, s);
+    case 16: return x_lines<16>(T, C, tab, out, tw, s);
+    case 32: return x_lines<32>(T, C, tab, out, tw, s);
+    case 64: return x_lines<64>(T, C, tab, out, tw, s);
+    case 128: return x_lines<128>(T, C, tab, out, tw, s);
+    case 256: return x_lines<256>(T, C, tab, out, tw, s);
+    case 512: return x_lines<512>(T, C, tab, out, tw, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t cols_dispatch(int P, double2 *data, long nbatch, long os, long rs, long ncols,
-                          const double2 *tw, cudaStream_t s) {
+cudaError_t y_dispatch(int P, const Tab &T, const Comps &C, int M, const double *in, double2 *out, const double2 *tw,
+                       cudaStream_t s) {
   switch (P) {
-    case 16: return cols_fft<16>(data, nbatch, os, rs, ncols, tw, s);
-    case 32: return cols_fft<32>(data, nbatch, os, rs, ncols, tw, s);
-    case 64: return cols_fft<64>(data, nbatch, os, rs, ncols, tw, s);
-    case 128: return cols_fft<128>(data, nbatch, os, rs, ncols, tw, s);
-    case 256: return cols_fft<256>(data, nbatch, os, rs, ncols, tw, s);
-    case 512: return cols_fft<512>(data, nbatch, os, rs, ncols, tw, s);
-    case 1024: return cols_fft<1024>(data, nbatch, os, rs, ncols, tw, s);
+    case 32: return y_cols<32>(T, C, M, in, out, tw, s);
+    case 64: return y_cols<64>(T, C, M, in, out, tw, s);
+    case 128: return y_cols<128>(T, C, M, in, out, tw, s);
+    case 256: return y_cols<256>(T, C, M, in, out, tw, s);
+    case 512: return y_cols<512>(T, C, M, in, out, tw, s);
+    case 1024: return y_cols<1024>(T, C, M, in, out, tw, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t z_dispatch(int P, int nz, long cols, int slots, const double2 *in, double *out, const double2 *tw,
+                       cudaStream_t s) {
+  switch (P) {
+    case 16: return z_cols<16>(nz, cols, slots, in, out, tw, s);
+    case 32: return z_cols<32>(nz, cols, slots, in, out, tw, s);
+    case 64: return z_cols<64>(nz, cols, slots, in, out, tw, s);
+    case 128: return z_cols<128>(nz, cols, slots, in, out, tw, s);
+    case 256: return z_cols<256>(nz, cols, slots, in, out, tw, s);
+    case 512: return z_cols<512>(nz, cols, slots, in, out, tw, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -496,13 +679,63 @@ CoefGeom coef_geom(const dds_ctx *ctx) {
 
 }  // namespace
 
+
+namespace {
+
+Box make_box(const double hb[3], const double t[3], double mu) {
+  const double dl = chord_length(hb, t);
+  return Box{0.5 * dl, mu * 0.31830988618379067154 * (hb[0] * hb[1] * hb[2]) / dl};
+}
+
+// Fields of one line direction (nf <= NF of them; the rest repeat the last).
+template <int NF>
+Fields<NF> make_fields(const CoefGeom &g, const double t[3], const double *b) {
+  Fields<NF> F;
+  F.t = v3(t[0], t[1], t[2]);
+  for (int f = 0; f < NF; ++f) {
+    const double *q = b + 3 * f;
+    F.b[f] = v3(q[0], q[1], q[2]);
+    F.w[f] = cross(F.b[f], F.t);
+  }
+  F.k1 = 1.0 / (1.0 - g.nu);
+  F.cell = make_box(g.h, t, g.mu);
+  F.sub = make_box(g.hs, t, g.mu);
+  return F;
+}
+
+// Table of NF fields (near: the stored near offsets, open boundary only).
+template <int NF>
+cudaError_t fill_table(const CoefGeom &g, const double t[3], const double *b, const Tab &T, int n_near,
+                       const int *d_near, double *tab, cudaStream_t s) {
+  const Fields<NF> F = make_fields<NF>(g, t, b);
+  const long N = tab_size(T);
+  if (g.n_shells > 2)                         // 49 images and more: a warp per offset
+    k_table_pbc<NF, 32><<<(unsigned)((N * 32 + 255) / 256), 256, 0, s>>>(g, F, T, tab);
+  else if (g.n_shells > 0)                    // 9 or 25 images
+    k_table_pbc<NF, 8><<<(unsigned)((N * 8 + 255) / 256), 256, 0, s>>>(g, F, T, tab);
+  else
+    k_table_far<NF><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(g, F, T, tab);
+  cudaError_t err = cudaGetLastError();
+  if (err == cudaSuccess && n_near > 0) {
+    k_table_near<NF><<<n_near, 128, 0, s>>>(g, F, T, d_near, tab);
+    err = cudaGetLastError();
+  }
+  return err;
+}
+
+// Consecutive effective fields whose tables are made together.
+struct Batch {
+  int e0, n, mx, my;
+};
+
+}  // namespace
+
 // -------------------------------------------------------------------------------
 cudaError_t launch_table_at(const CoefGeom &g, const double t[3], const double b[3], long n,
                             const int *d_ijk, double *d_out, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int nt = 128;
-  k_table_at<<<(unsigned)((n + nt - 1) / nt), nt, 0, s>>>(g, v3(t[0], t[1], t[2]), v3(b[0], b[1], b[2]),
-                                                           n, d_ijk, d_out);
+  k_table_at<<<(unsigned)((n + nt - 1) / nt), nt, 0, s>>>(g, make_fields<1>(g, t, b), n, d_ijk, d_out);
   return cudaGetLastError();
 }
 
@@ -511,12 +744,61 @@ CoefGeom make_coef_geom(const dds_ctx *ctx) { return coef_geom(ctx); }
 int build_spectra(dds_ctx *ctx, cudaStream_t s) {
   const Shape &sh = ctx->shape;
   const int px = 2 * sh.M, py = sh.py, pz = sh.pz, M = sh.M;
-  const long P = (long)px * py * pz;
-  const long nspec = (long)(M + 1) * py * pz;
+  const size_t P = (size_t)px * py * pz;
   const CoefGeom g = coef_geom(ctx);
+  const double *ft = ctx->field_t.data(), *fb = ctx->field_b.data();
 
-  // near offsets (decided on the host, same expression as the definition)
+  // workspace: at most what a full padded FP64 table of one field and one complex
+  // spectrum take (or 1 GB): fields of one direction share a table, and as many
+  // components as fit share a launch
+  const size_t limit = std::max((size_t)1 << 30, 48 * P + 16 * (size_t)(M + 1) * py * pz);
+  auto tab_of = [&](int mx, int my) {
+    Tab T;
+    T.nx = sh.nx;
+    T.ny = sh.ny;
+    T.nz = sh.nz;
+    T.mx = mx;
+    T.my = my;
+    T.rx = mx ? sh.nx : 2 * sh.nx - 1;
+    T.ry = (my || py == sh.ny) ? sh.ny : 2 * sh.ny - 1;      // periodic in y: rows 0 .. ny - 1
+    return T;
+  };
+  auto slot_bytes = [&](const Tab &T, size_t *x, size_t *y, size_t *z) {
+    const size_t ky = T.mx ? py / 2 + 1 : py, c = M + 1;
+    *x = (size_t)T.nz * T.ry * c * (T.mx ? 8 : 16);
+    *y = (size_t)T.nz * ky * c * 16;
+    *z = (size_t)pz * ky * c * 8;
+  };
+  std::vector<Batch> batches;
+  size_t tab_max = 0, buf1_max = 0, buf2_max = 0;
+  std::vector<int> slots_of;
+  for (int e = 0; e < ctx->fe;) {
+    auto flag = [&](int q, int a) { return mirror_ok(ft + 3 * q, fb + 3 * q, a) ? 1 : 0; };
+    Batch b{e, 1, flag(e, 0), flag(e, 1)};
+    while (b.n < 3 && e + b.n < ctx->fe && flag(e + b.n, 0) == b.mx && flag(e + b.n, 1) == b.my &&
+           ft[3 * e] == ft[3 * (e + b.n)] && ft[3 * e + 1] == ft[3 * (e + b.n) + 1] &&
+           ft[3 * e + 2] == ft[3 * (e + b.n) + 2])
+      ++b.n;
+    const Tab T = tab_of(b.mx, b.my);
+    size_t x, y, z;
+    slot_bytes(T, &x, &y, &z);
+    const int least = b.mx ? 2 : 1;
+    int slots = 6;
+    auto total = [&]() { return 48 * (size_t)b.n * tab_size(T) + slots * (std::max(x, z) + y); };
+    while (total() > limit && slots > least) slots = slots > 2 ? 2 : least;
+    while (total() > limit && b.n > 1) --b.n;
+    batches.push_back(b);
+    slots_of.push_back(slots);
+    tab_max = std::max(tab_max, 48 * (size_t)b.n * tab_size(T));
+    buf1_max = std::max(buf1_max, slots * std::max(x, z));
+    buf2_max = std::max(buf2_max, slots * y);
+    e += b.n;
+  }
+
+  // near offsets the tables hold (decided on the host, same expression as the
+  // definition): all of them, then those with i >= 0, j >= 0 and both, by (mx, my)
   std::vector<int> near;                 // with replica shells the table kernel handles them
+  int near_at[2][2] = {{0, 0}, {0, 0}}, near_n[2][2] = {{0, 0}, {0, 0}};
   if (ctx->n_near > 0.0 && ctx->n_shells == 0) {
     double hmax = fmax(ctx->h[0], fmax(ctx->h[1], ctx->h[2]));
     int lim[3] = {ctx->nx - 1, ctx->ny - 1, ctx->nz - 1};
@@ -524,80 +806,123 @@ int build_spectra(dds_ctx *ctx, cudaStream_t s) {
       const double c = ceil(ctx->n_near * hmax / ctx->h[a]) + 1.0;
       if (c < lim[a]) lim[a] = (int)c;
     }
-    for (int k = -lim[2]; k <= lim[2]; ++k)
-      for (int j = -lim[1]; j <= lim[1]; ++j)
-        for (int i = -lim[0]; i <= lim[0]; ++i)
-          if (is_near(ctx->h, ctx->n_near, i, j, k)) {
-            near.push_back(i);
-            near.push_back(j);
-            near.push_back(k);
-          }
+    for (int mx = 0; mx < 2; ++mx)
+      for (int my = 0; my < 2; ++my) {
+        bool used = false;
+        for (const Batch &b : batches) used = used || (b.mx == mx && b.my == my);
+        if (!used) continue;
+        near_at[mx][my] = (int)near.size();
+        for (int k = 0; k <= lim[2]; ++k)
+          for (int j = my ? 0 : -lim[1]; j <= lim[1]; ++j)
+            for (int i = mx ? 0 : -lim[0]; i <= lim[0]; ++i)
+              if (is_near(ctx->h, ctx->n_near, i, j, k)) {
+                near.push_back(i);
+                near.push_back(j);
+                near.push_back(k);
+              }
+        near_n[mx][my] = ((int)near.size() - near_at[mx][my]) / 3;
+      }
   }
-  const int n_near = (int)(near.size() / 3);
 
-  double *tab = nullptr;
-  double2 *spec = nullptr;
+  double *tab = nullptr, *buf1 = nullptr;
+  double2 *buf2 = nullptr;
   int *d_near = nullptr;
   unsigned long long *d_amax = nullptr;
-  cudaError_t err = cudaMallocAsync(&tab, sizeof(double) * 6 * P, s);
+  cudaError_t err = cudaMallocAsync(&tab, tab_max, s);
   if (err == cudaSuccess) err = cudaMallocAsync(&d_amax, sizeof(unsigned long long), s);
-  if (err == cudaSuccess) err = cudaMallocAsync(&spec, sizeof(double2) * nspec, s);
-  if (err == cudaSuccess && n_near > 0) err = cudaMallocAsync(&d_near, sizeof(int) * 3 * n_near, s);
+  if (err == cudaSuccess) err = cudaMallocAsync(&buf1, buf1_max, s);
+  if (err == cudaSuccess) err = cudaMallocAsync(&buf2, buf2_max, s);
+  if (err == cudaSuccess && !near.empty()) err = cudaMallocAsync(&d_near, sizeof(int) * near.size(), s);
   if (err != cudaSuccess) {
     cudaFreeAsync(tab, s);
-    cudaFreeAsync(spec, s);
+    cudaFreeAsync(buf1, s);
+    cudaFreeAsync(buf2, s);
     cudaFreeAsync(d_near, s);
     cudaFreeAsync(d_amax, s);
     cudaGetLastError();
     return fail(ctx, DDS_ERR_OOM, "build_kernels: cannot allocate %.2f GB of FP64 table workspace: %s",
-                (sizeof(double) * 6.0 * P + sizeof(double2) * (double)nspec) / 1e9, cudaGetErrorString(err));
+                (double)(tab_max + buf1_max + buf2_max) / 1e9, cudaGetErrorString(err));
   }
-  if (n_near > 0)
-    err = cudaMemcpyAsync(d_near, near.data(), sizeof(int) * 3 * n_near, cudaMemcpyHostToDevice, s);
+  if (!near.empty())
+    err = cudaMemcpyAsync(d_near, near.data(), sizeof(int) * near.size(), cudaMemcpyHostToDevice, s);
 
   const double scale = 1.0 / ((double)px * (double)py * (double)pz);
-  for (int e = 0; e < ctx->fe && err == cudaSuccess; ++e) {
-    const V3 t = v3(ctx->field_t[3 * e], ctx->field_t[3 * e + 1], ctx->field_t[3 * e + 2]);
-    const V3 b = v3(ctx->field_b[3 * e], ctx->field_b[3 * e + 1], ctx->field_b[3 * e + 2]);
-    k_table_far<<<(unsigned)((P + 255) / 256), 256, 0, s>>>(g, t, b, ctx->nx, ctx->ny, ctx->nz, px, py,
-                                                             pz, tab);
-    err = cudaGetLastError();
-    if (err == cudaSuccess && n_near > 0) {
-      k_table_near<<<n_near, 128, 0, s>>>(g, t, b, px, py, pz, d_near, tab);
-      err = cudaGetLastError();
-    }
-    for (int c = 0; c < 6 && err == cudaSuccess; ++c) {
-      err = r2c_dispatch(M, tab + c * P, (long)py * pz, spec, ctx->tw.f64, s);
-      if (err == cudaSuccess)   // y: batches kz, rows ky (pitch M+1), columns kx
-        err = cols_dispatch(py, spec, pz, (long)py * (M + 1), M + 1, M + 1, ctx->tw.f64, s);
-      if (err == cudaSuccess)   // z: one batch, rows kz, columns (ky, kx)
-        err = cols_dispatch(pz, spec, 1, 0, (long)py * (M + 1), (long)py * (M + 1), ctx->tw.f64, s);
-      if (err == cudaSuccess) {
-        const long n = sh.zfour ? zf_stored_tiles(sh) * pz * sh.wz : (long)py * (M + 1) * pz;
-        const unsigned blocks = (unsigned)((n + 255) / 256);
-        if (ctx->spectra_fp16) {
-          err = cudaMemsetAsync(d_amax, 0, sizeof(unsigned long long), s);
-          if (err == cudaSuccess) {
-            k_absmax_imag<<<1024, 256, 0, s>>>(spec, nspec, d_amax);
-            k_store_scale<<<1, 1, 0, s>>>(d_amax, scale, ctx->kscale, c * sh.fe + e);
-            __half *out = static_cast<__half *>(ctx->kspec);
-            if (sh.zfour) k_extract_four<__half><<<blocks, 256, 0, s>>>(spec, sh, e, c, scale, d_amax, out);
-            else k_extract<__half><<<blocks, 256, 0, s>>>(spec, M, py, pz, sh.wz, sh.zreg_g, sh.fe, e, c, scale,
-                                                          d_amax, out);
+  for (size_t ib = 0; ib < batches.size() && err == cudaSuccess; ++ib) {
+    const Batch &b = batches[ib];
+    const Tab T = tab_of(b.mx, b.my);
+    const double *t = ft + 3 * b.e0, *bv = fb + 3 * b.e0;
+    const int nn = near_n[b.mx][b.my];
+    const int *dn = d_near + near_at[b.mx][b.my];
+    if (b.n == 1) err = fill_table<1>(g, t, bv, T, nn, dn, tab, s);
+    else if (b.n == 2) err = fill_table<2>(g, t, bv, T, nn, dn, tab, s);
+    else err = fill_table<3>(g, t, bv, T, nn, dn, tab, s);
+    for (int f = 0; f < b.n && err == cudaSuccess; ++f) {
+      const int e = b.e0 + f;
+      Comps all{};
+      all.off = 6 * f;
+      for (int c = 0; c < 6; ++c) {
+        all.sx[c] = b.mx ? mirror_parity(fb + 3 * e, 0, c) : 1;
+        all.sy[c] = b.my ? mirror_parity(fb + 3 * e, 1, c) : 1;
+      }
+      // line sets: with the x mirror each x-odd component shares the line of an x-even one
+      std::vector<std::pair<int, int>> sets;
+      std::vector<int> even, odd;
+      for (int c = 0; c < 6; ++c) (b.mx && all.sx[c] < 0 ? odd : even).push_back(c);
+      for (size_t q = 0; q < std::max(even.size(), odd.size()); ++q) {
+        if (q >= even.size()) sets.push_back({odd[q], -1});
+        else sets.push_back({even[q], q < odd.size() ? odd[q] : -1});
+      }
+      const size_t cols = (size_t)(b.mx ? py / 2 + 1 : py) * (M + 1);
+      for (size_t q = 0; q < sets.size() && err == cudaSuccess;) {
+        Comps C = all;
+        for (; q < sets.size(); ++q) {
+          const int add = sets[q].second >= 0 ? 2 : 1;
+          if (C.slots + add > slots_of[ib]) break;
+          C.ce[C.sets] = sets[q].first;
+          C.co[C.sets] = sets[q].second;
+          C.se[C.sets] = C.slots;
+          C.comp_of[C.slots++] = sets[q].first;
+          C.so[C.sets] = 0;
+          if (add == 2) {
+            C.so[C.sets] = C.slots;
+            C.comp_of[C.slots++] = sets[q].second;
+          }
+          ++C.sets;
+        }
+        err = x_dispatch(M, T, C, tab, buf1, ctx->tw.f64, s);
+        if (err == cudaSuccess) err = y_dispatch(py, T, C, M, buf1, buf2, ctx->tw.f64, s);
+        if (err == cudaSuccess) err = z_dispatch(pz, T.nz, (long)cols, C.slots, buf2, buf1, ctx->tw.f64, s);
+        for (int slot = 0; slot < C.slots && err == cudaSuccess; ++slot) {
+          const int c = C.comp_of[slot];
+          const double *spec = buf1 + (size_t)slot * pz * cols;
+          const int fold = b.mx ? -C.sx[c] : 0;
+          const long n = sh.zfour ? zf_stored_tiles(sh) * pz * sh.wz : (long)py * (M + 1) * pz;
+          const unsigned blocks = (unsigned)((n + 255) / 256);
+          if (ctx->spectra_fp16) {
+            err = cudaMemsetAsync(d_amax, 0, sizeof(unsigned long long), s);
+            if (err == cudaSuccess) {
+              k_absmax_imag<<<1024, 256, 0, s>>>(spec, (long)(pz * cols), d_amax);
+              k_store_scale<<<1, 1, 0, s>>>(d_amax, scale, ctx->kscale, c * sh.fe + e);
+              __half *out = static_cast<__half *>(ctx->kspec);
+              if (sh.zfour) k_extract_four<__half><<<blocks, 256, 0, s>>>(spec, fold, sh, e, c, scale, d_amax, out);
+              else k_extract<__half><<<blocks, 256, 0, s>>>(spec, fold, M, py, pz, sh.wz, sh.zreg_g, sh.fe, e, c,
+                                                            scale, d_amax, out);
+              err = cudaGetLastError();
+            }
+          } else {
+            float *out = static_cast<float *>(ctx->kspec);
+            if (sh.zfour) k_extract_four<float><<<blocks, 256, 0, s>>>(spec, fold, sh, e, c, scale, nullptr, out);
+            else k_extract<float><<<blocks, 256, 0, s>>>(spec, fold, M, py, pz, sh.wz, sh.zreg_g, sh.fe, e, c, scale,
+                                                         nullptr, out);
             err = cudaGetLastError();
           }
-        } else {
-          float *out = static_cast<float *>(ctx->kspec);
-          if (sh.zfour) k_extract_four<float><<<blocks, 256, 0, s>>>(spec, sh, e, c, scale, nullptr, out);
-          else k_extract<float><<<blocks, 256, 0, s>>>(spec, M, py, pz, sh.wz, sh.zreg_g, sh.fe, e, c, scale,
-                                                       nullptr, out);
-          err = cudaGetLastError();
         }
       }
     }
   }
   cudaFreeAsync(tab, s);
-  cudaFreeAsync(spec, s);
+  cudaFreeAsync(buf1, s);
+  cudaFreeAsync(buf2, s);
   cudaFreeAsync(d_near, s);
   cudaFreeAsync(d_amax, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);

@@ -67,6 +67,11 @@ __host__ __device__ inline long zf_stored_tiles(const Shape &sh) {
 // the number of kernel-spectrum values the three-stage z pass stores.
 size_t zfour_symmetry(const double *field_t, const double *field_b, int fe, Shape *sh);
 
+// Whether the mirror x_a -> -x_a maps the segment of (t, b) onto itself and b onto +-b,
+// and the parity of component c (xx, yy, zz, xy, xz, yz) of its coefficients under it.
+bool mirror_ok(const double *t, const double *b, int a);
+int mirror_parity(const double *b, int a, int c);
+
 // FP64 description of a box coefficient (Eq. 9b times the cell volume).
 struct CoefGeom {
   double h[3];        // cell edges
