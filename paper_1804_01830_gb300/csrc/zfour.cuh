@@ -132,27 +132,32 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
   const long st = nyq ? (long)(sh.zs.xall ? py / 2 + 1 : py) * ktiles + nyq_idx
                       : (long)(sw ? py - ky : ky) * ktiles + kxt;
   const GT *ks = kspec + st * 6L * FE * PZ * W;
-  // the tile's kernel spectra (6 FE PZ W values, contiguous) head for L2 now, so the
+  // the tile's kernel spectra (6 FE PZ W values, contiguous) head for L2, so the
   // per-component loads of stage 2 find them there; a negated-frequency tile leaves
   // them to its partner launched beside it
-  if (!sw) {
+  auto prefetch_spectra = [&]() {
     constexpr unsigned BYTES = 6u * FE * PZ * W * sizeof(GT), CH = 8192, NCH = (BYTES + CH - 1) / CH;
     static_assert(BYTES % 16 == 0 && NCH <= NT, "prefetch chunks");
-    if (tid < (int)NCH) prefetch_l2_bulk(reinterpret_cast<const char *>(ks) + tid * CH, min(CH, BYTES - tid * CH));
-  }
+    if (!sw && tid < (int)NCH)
+      prefetch_l2_bulk(reinterpret_cast<const char *>(ks) + tid * CH, min(CH, BYTES - tid * CH));
+  };
 
   // stage 1: forward R1-point DFTs over n1 of the rows n2 + 8 n1 (n1 < R1/2 non-zero);
   // a negated-frequency tile transforms -s_b conj(rho) (s_b folds the spectra's sign)
   constexpr int NI = FE * R2 * W;              // items (field, n2, column)
+  // element (e, z, w) of the tile's rows: src[e se + z sz + w sw1].  One pointer for both
+  // kinds of tile: a choice between two loads per element compiles to branches, which
+  // keep the loads of an item from being in flight together (padded z 128, 512x512x64
+  // with two sets: 5.14 -> 3.21 ms)
+  const float2 *src = nyq ? in_nyq + (long)nyq_idx * W * nz : in_main + (long)ky * M + kxt * W;
+  const long sz = nyq ? 1 : (long)py * M, sw1 = nyq ? nz : 1, se = (long)nz * py * (nyq ? 1 : M);
   auto s1_load = [&](int item, float2 (&ev)[H]) {
     const int e = item / (R2 * W), r = item - e * (R2 * W), n2 = r / W, w = r - n2 * W;
+    const float2 *p = src + e * se + n2 * sz + w * sw1;
 #pragma unroll
     for (int n1 = 0; n1 < H; ++n1) {
-      const int z = n2 + R2 * n1;
       ev[n1] = make_float2(0.f, 0.f);
-      if (z < nz)
-        ev[n1] = !nyq ? __ldg(in_main + (((long)e * nz + z) * py + ky) * M + kxt * W + w)
-                      : __ldg(in_nyq + ((long)e * py + nyq_idx * W + w) * nz + z);
+      if (n2 + R2 * n1 < nz) ev[n1] = __ldg(p + n1 * (R2 * sz));
     }
   };
   auto s1_finish = [&](int item, float2 (&ev)[H]) {
@@ -181,6 +186,9 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
     const bool two = item + NT < NI;
     s1_load(item, a);
     if (two) s1_load(item + NT, b);
+    // the rows first: requested ahead of them, the spectra delay them (GaN layer, with the
+    // single pointer: 1.04 -> 0.93 ms)
+    if (item == tid) prefetch_spectra();
     s1_finish(item, a);
     if (two) s1_finish(item + NT, b);
   }
@@ -245,6 +253,8 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
     }
     dft_reg<H, true>(ev);
     dft_reg<H, true>(od);
+    float2 *dst = nyq ? out_nyq + ((long)c * py + nyq_idx * W + wc) * nz
+                      : out_main + ((long)c * nz * py + ky) * M + kxt * W + wc;
 #pragma unroll
     for (int b = 0; b < H; ++b) {
       const int z = a + R2 * b;
@@ -255,8 +265,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
         // and they leave L2 to the mirror tiles' spectra (1.049 -> 1.041 ms); streaming
         // loads of the density rows cost more (1.088 ms), since neighbouring tiles share
         // their 128-byte lines
-        if (!nyq) __stcs(out_main + (((long)c * nz + z) * py + ky) * M + kxt * W + wc, v);
-        else __stcs(out_nyq + ((long)c * py + nyq_idx * W + wc) * nz + z, v);
+        __stcs(dst + z * sz, v);
       }
     }
   }

@@ -292,6 +292,11 @@ __global__ void __launch_bounds__(128) k_zreg(Shape sh, const float2 *in_main, c
   }
   const float2 *twP = tw + tw_offset(P);
 
+  // rows z of this lane's column in the inputs and outputs: one pointer and stride for
+  // both kinds of tile, so that all loads are in flight together
+  const long sz = nyq ? 1 : (long)py * M, se = (long)nz * py * (nyq ? 1 : M);
+  const float2 *src = nyq ? in_nyq + ky * nz : in_main + ky * M + kx;
+  float2 *dst = nyq ? out_nyq + ky * nz : out_main + ky * M + kx;
   float2 f[FE][E];
 #pragma unroll
   for (int e = 0; e < FE; ++e) {
@@ -299,13 +304,8 @@ __global__ void __launch_bounds__(128) k_zreg(Shape sh, const float2 *in_main, c
     for (int m = 0; m < E; ++m) f[e][m] = make_float2(0.f, 0.f);
     if (e < fe) {
 #pragma unroll
-      for (int m = 0; m < E / 2; ++m) {
-        const int z = g + G * m;
-        if (z < nz) {
-          f[e][m] = !nyq ? __ldg(in_main + (((long)e * nz + z) * py + ky) * M + kx)
-                         : __ldg(in_nyq + ((long)e * py + ky) * nz + z);
-        }
-      }
+      for (int m = 0; m < E / 2; ++m)
+        if (g + G * m < nz) f[e][m] = __ldg(src + e * se + (g + G * m) * sz);
     }
   }
   // kernel spectra of component 0, in flight while the fields are transformed
@@ -364,10 +364,7 @@ __global__ void __launch_bounds__(128) k_zreg(Shape sh, const float2 *in_main, c
 #pragma unroll
     for (int m = 0; m < E / 2; ++m) {
       const int z = g + G * m;
-      if (z < nz) {
-        if (!nyq) out_main[(((long)c * nz + z) * py + ky) * M + kx] = s[m];
-        else out_nyq[((long)c * py + ky) * nz + z] = s[m];
-      }
+      if (z < nz) dst[c * se + z * sz] = s[m];
     }
   }
 }
