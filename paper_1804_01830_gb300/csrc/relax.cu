@@ -16,6 +16,7 @@
 // so every quantity the kernels touch is in units of u.  One step reads u and
 // dt f and writes u: 36 bytes per cell from HBM.
 #include <algorithm>
+#include <type_traits>
 
 #include "dds_internal.h"
 
@@ -28,6 +29,7 @@ struct RelaxCoef {
   //                          + sum_{b != a} mix[a][b] (4-point cross of u_b in a, b)
   float lap[3][3];
   float mix[3][3];
+  float2 lap2[3][3], mix2[3][3];   // the same twice, for packed pairs of cells
   // ghost layers: first derivatives 1/(2 h) and the factors of Eq. 18b
   float inv2h[3];
   float two_dz;      // 2 dz
@@ -45,34 +47,6 @@ __device__ __forceinline__ int wrap(int i, int n) { return i < 0 ? i + n : (i >=
 
 __device__ __forceinline__ long cidx(const RelaxCoef &r, int c, int k, int j, int i) {
   return (((long)c * r.nz + k) * r.ny + j) * r.nx + i;
-}
-
-// u_c at film cell (i, j, k) with i, j periodic and k in [-1, nz]: the ghost layers of
-// Eq. 18b below (k = -1) and above (k = nz).  phi: [surface][3][ny][nx].
-__device__ __forceinline__ float uext(const RelaxCoef &r, const float *__restrict__ u, const float *__restrict__ phi, int c,
-                      int i, int j, int k) {
-  i = wrap(i, r.nx);
-  j = wrap(j, r.ny);
-  if (k >= 0 && k < r.nz) return __ldg(u + cidx(r, c, k, j, i));
-  const bool top = k >= r.nz;
-  const int ks = top ? r.nz - 1 : 0;          // surface layer (centre of the condition)
-  const int kn = top ? r.nz - 2 : 1;          // its inner neighbour
-  const float sgn = top ? 1.f : -1.f;         // ghost = inner + sgn * 2dz * (condition terms)
-  const float *ph = phi + (long)(top ? 3 : 0) * r.ny * r.nx + (long)j * r.nx + i;
-  const long plane = (long)r.ny * r.nx;
-  const float inner = __ldg(u + cidx(r, c, kn, j, i));
-  if (c == 0) {   // (du_x/dz + du_z/dx) / 2 = phi_xz
-    const float dxuz = (__ldg(u + cidx(r, 2, ks, j, wrap(i + 1, r.nx))) - __ldg(u + cidx(r, 2, ks, j, wrap(i - 1, r.nx)))) * r.inv2h[0];
-    return inner + sgn * r.two_dz * (2.f * __ldg(ph) - dxuz);
-  }
-  if (c == 1) {   // (du_y/dz + du_z/dy) / 2 = phi_yz
-    const float dyuz = (__ldg(u + cidx(r, 2, ks, wrap(j + 1, r.ny), i)) - __ldg(u + cidx(r, 2, ks, wrap(j - 1, r.ny), i))) * r.inv2h[1];
-    return inner + sgn * r.two_dz * (2.f * __ldg(ph + plane) - dyuz);
-  }
-  // (1 - nu) du_z/dz + nu (du_x/dx + du_y/dy) = phi_zz
-  const float dxux = (__ldg(u + cidx(r, 0, ks, j, wrap(i + 1, r.nx))) - __ldg(u + cidx(r, 0, ks, j, wrap(i - 1, r.nx)))) * r.inv2h[0];
-  const float dyuy = (__ldg(u + cidx(r, 1, ks, wrap(j + 1, r.ny), i)) - __ldg(u + cidx(r, 1, ks, wrap(j - 1, r.ny), i))) * r.inv2h[1];
-  return inner + sgn * r.zfac * (__ldg(ph + 2 * plane) - r.nu * (dxux + dyuy));
 }
 
 // dt f (Eq. 15) at every film cell and phi (Eq. 16c) on the two surface layers.
@@ -110,144 +84,313 @@ __global__ void k_relax_prep(RelaxCoef r, const float *__restrict__ sig, float *
   }
 }
 
-// One explicit step, u_out = u_in + dt (navier(u_in) + f), on a tile of TX x TY columns
-// marching up a chunk of KZ layers: three planes (below, at, above the layer) of all
-// three components, with a one-cell halo, rotate through shared memory, so every value
-// of u is read from global memory about once per step (halo cells from L2).  The plane
-// two layers ahead is loaded into registers while the current layer is updated; ghost
-// planes are evaluated (uext) as they are loaded.
-// (32-layer chunks: each chunk restarts its march with three plane loads; GaN grid
-// 0.0986 -> 0.0948 ms per step against 16-layer chunks; 32x16 and 64x8 tiles were slower)
-constexpr int TX = 32, TY = 8, KZ = 32, HX = TX + 2, HY = TY + 2;
-constexpr int NT_TILE = TX * TY, PLANE = 3 * HY * HX, NQ = (PLANE + NT_TILE - 1) / NT_TILE;
+// The march over the film, shared by the step and the stress kernels.  256 threads take a
+// tile of 64 x 8 columns, two x-adjacent cells per thread, up a chunk of layers.  Planes of
+// u (three components, one-cell halo) arrive in a ring of shared-memory slots by
+// cp.async, up to three layers ahead of the layer that uses them; ghost planes are evaluated
+// into their slot.  A plane is read from shared memory once, when it is the one above the
+// current layer: every term of the operator is a combination of in-plane terms of the
+// layer's own plane and of differences between the planes above and below, so a thread
+// carries the centre values, four in-plane differences and the in-plane part of the
+// operator in registers.  That is 12 shared-memory loads per cell against 45 with three
+// resident planes, and one barrier per layer against two.  The march is unrolled by three:
+// the carried terms then stay in fixed registers.  The two
+// cells' arithmetic is packed (add/fma on pairs of FP32).  FULL: rows are whole tiles and everything is aligned, so no
+// access is predicated.  What bounds it: shared-memory wavefronts (about half the time) and
+// the latency of a layer's chain at two CTAs per SM (their registers), with DRAM at half its
+// rate; deeper rings and one cell per thread measured the same or slower.  Step, GaN grid
+// 256x256x128: 94 -> 77 us, 512x512x16: 61 -> 49 us; total stress: 442 -> 105 us and 226 ->
+// 63 us (it evaluated ghost layers and offsets per value before).
+constexpr int TX = 64, TY = 8, PX = TX / 2, HY = TY + 2, NTM = PX * TY, RING = 4;
+constexpr int X0 = 4, LD = TX + 8;                 // column x of the tile at X0 + x: 16-byte aligned rows
+constexpr int CS = HY * LD, PLANE = 3 * CS;
+// a slot: one plane, and the threads' own inputs (NC fields) of the layer below it
+template <int NC> __host__ __device__ constexpr int slot_floats() { return PLANE + NC * 2 * NTM; }
 
 __device__ __forceinline__ int mod(int i, int n) { return ((i % n) + n) % n; }
 
-// The values of one plane (layer k, or a ghost layer) this thread stages: entry q of
-// the [component][y][x] halo tile for q = threadIdx.x + NT_TILE * e, whose film
-// element is u[base[e] + k * plane] (32-bit offsets: 3 nx ny nz < 2^31 for every grid
-// the library accepts).
-__device__ __forceinline__ void fetch_plane(const RelaxCoef &r, const float *__restrict__ u,
-                                            const float *__restrict__ phi, const int (&base)[NQ], const int (&comp)[NQ],
-                                            int k, int plane, float (&v)[NQ]) {
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+__device__ __forceinline__ void cp_async4(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8f(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async16f(float *dst, const float *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// The part of every plane one thread stages: two groups of four columns and, for the first
+// threads, one halo column, as offsets of the film element in layer 0 and of the slot
+// element (fixed for the whole march; source -1: none).
+struct Stage {
+  int src[3], dst[3];
+  int col;                 // first column of the groups
+};
+__device__ __forceinline__ Stage make_stage(const RelaxCoef &r, int i0, int j0) {
+  constexpr int G = TX / 4, ROWS = 3 * HY, PASS = NTM / G;
+  static_assert(ROWS <= 2 * PASS && 2 * ROWS <= NTM, "two passes over the rows, one over the halo columns");
+  auto film = [&](int row, int i) { return (int)cidx(r, row / HY, 0, mod(j0 + row % HY - 1, r.ny), i); };
+  Stage st;
+  const int x = 4 * (threadIdx.x % G);
+  st.col = i0 + x;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    const int row = threadIdx.x / G + PASS * e;
+    st.src[e] = row < ROWS && st.col <= r.nx ? film(row, st.col) : -1;   // column nx is the last that is read
+    st.dst[e] = row * LD + X0 + x;
+  }
+  const int row = threadIdx.x >> 1, hx = threadIdx.x & 1 ? TX : -1;
+  st.src[2] = row < ROWS && i0 + hx <= r.nx ? film(row, mod(i0 + hx, r.nx)) : -1;
+  st.dst[2] = row * LD + X0 + hx;
+  return st;
+}
+
+// Ghost plane k = -1 or nz of a tile and its halo (Eq. 18b and its counterparts) into slot
+// pl: the inner neighbour of the surface layer plus or minus 2 dz times
+//   u_x: 2 phi_xz - du_z/dx,  u_y: 2 phi_yz - du_z/dy,
+//   u_z: (phi_zz - nu (du_x/dx + du_y/dy)) / (1 - nu).  A thread evaluates
+// all components at its three positions with every load in flight: one position and
+// component at a time, the surface chunks waited 8 times a memory latency for it.
+__device__ __forceinline__ void ghost_plane(const RelaxCoef &r, const float *__restrict__ u,
+                                            const float *__restrict__ phi, int i0, int j0, int k, float *pl) {
+  constexpr int W = TX + 2, NP = (HY * W + NTM - 1) / NTM;
+  const bool top = k >= r.nz;
+  const int plane = r.ny * r.nx, cs = r.nz * plane;
+  const float *us = u + (top ? r.nz - 1 : 0) * plane, *un = u + (top ? r.nz - 2 : 1) * plane;
+  const float *ph = phi + (top ? 3 : 0) * plane;
+  const float sgn = top ? 1.f : -1.f;
+  float in[NP][3], f[NP][3], zx[NP][2], zy[NP][2], xx[NP][2], yy[NP][2];
+#pragma unroll
+  for (int e = 0; e < NP; ++e) {
+    const int p = threadIdx.x + NTM * e, hy = p / W, x = i0 + p - hy * W - 1;
+    const bool used = p < HY * W && x <= r.nx;     // column nx is the last that is read
+    const int i = used ? wrap(x, r.nx) : 0, j = used ? mod(j0 + hy - 1, r.ny) : 0;
+    const int o = j * r.nx + i, oe = j * r.nx + wrap(i + 1, r.nx), ow = j * r.nx + wrap(i - 1, r.nx);
+    const int on = wrap(j + 1, r.ny) * r.nx + i, os = wrap(j - 1, r.ny) * r.nx + i;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      in[e][c] = __ldg(un + c * cs + o);
+      f[e][c] = __ldg(ph + c * plane + o);
+    }
+    zx[e][0] = __ldg(us + 2 * cs + oe);
+    zx[e][1] = __ldg(us + 2 * cs + ow);
+    zy[e][0] = __ldg(us + 2 * cs + on);
+    zy[e][1] = __ldg(us + 2 * cs + os);
+    xx[e][0] = __ldg(us + oe);
+    xx[e][1] = __ldg(us + ow);
+    yy[e][0] = __ldg(us + cs + on);
+    yy[e][1] = __ldg(us + cs + os);
+  }
+#pragma unroll
+  for (int e = 0; e < NP; ++e) {
+    const int p = threadIdx.x + NTM * e, hy = p / W, x = p - hy * W - 1;
+    if (p >= HY * W || i0 + x > r.nx) continue;
+    float *d = pl + hy * LD + X0 + x;
+    d[0] = in[e][0] + sgn * r.two_dz * (2.f * f[e][0] - (zx[e][0] - zx[e][1]) * r.inv2h[0]);
+    d[CS] = in[e][1] + sgn * r.two_dz * (2.f * f[e][1] - (zy[e][0] - zy[e][1]) * r.inv2h[1]);
+    d[2 * CS] = in[e][2] + sgn * r.zfac * (f[e][2] - r.nu * ((xx[e][0] - xx[e][1]) * r.inv2h[0] + (yy[e][0] - yy[e][1]) * r.inv2h[1]));
+  }
+}
+
+// Starts plane k (a layer, or a ghost layer at -1 and nz) into slot pl, in the current copy group.
+// vec: rows of u are 16-byte aligned (whole groups of four).
+template <bool FULL>
+__device__ __forceinline__ void start_plane(const RelaxCoef &r, const float *__restrict__ u,
+                                            const float *__restrict__ phi, const Stage &st, int i0, int j0, int k,
+                                            bool vec, float *pl) {
   if (k >= 0 && k < r.nz) {
-    const int kp = k * plane;
+    const float *layer = u + (long)k * (r.ny * r.nx);
+    if constexpr (FULL) {
+      cp_async16f(pl + st.dst[0], layer + st.src[0]);
+      if (st.src[1] >= 0) cp_async16f(pl + st.dst[1], layer + st.src[1]);
+    } else {
 #pragma unroll
-    for (int e = 0; e < NQ; ++e)
-      if (comp[e] >= 0) v[e] = __ldg(u + base[e] + kp);
+      for (int e = 0; e < 2; ++e) {
+        if (st.src[e] < 0) continue;
+        const float *src = layer + st.src[e];
+        float *dst = pl + st.dst[e];
+        if (vec && st.col < r.nx) {
+          cp_async16f(dst, src);
+          if (st.col + 4 == r.nx) cp_async4(dst + 4, src + 4 - r.nx);    // a row that ends inside the tile: its halo
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {            // past the last column: the first again
+            const int i = st.col + q;
+            if (i <= r.nx) cp_async4(dst + q, src + q - (i == r.nx ? r.nx : 0));
+          }
+        }
+      }
+    }
+    if (st.src[2] >= 0) cp_async4(pl + st.dst[2], layer + st.src[2]);
   } else {
-#pragma unroll
-    for (int e = 0; e < NQ; ++e) {
-      if (comp[e] < 0) continue;
-      const int col = base[e] - comp[e] * r.nz * plane;
-      const int j = col / r.nx, i = col - j * r.nx;
-      v[e] = uext(r, u, phi, comp[e], i, j, k);
-    }
+    ghost_plane(r, u, phi, i0, j0, k, pl);
   }
 }
 
-__device__ __forceinline__ void store_plane(const float (&v)[NQ], const int (&comp)[NQ], float *pl) {
-#pragma unroll
-  for (int e = 0; e < NQ; ++e)
-    if (comp[e] >= 0) pl[threadIdx.x + NT_TILE * e] = v[e];
+// What a thread keeps of a plane for its two cells: centre values; u_x(x+1) - u_x(x-1) and
+// the same of u_z; u_y(y+1) - u_y(y-1) and the same of u_z.  STEP: in[a] = the in-plane
+// part of the operator; otherwise in[0], in[1] = the x difference of u_y and the y
+// difference of u_x.
+struct PlaneTerms {
+  float2 c[3], ax, az, by, bz, in[3];
+};
+
+// The values at x (the two cells), x - 1 and x + 1 of one row.
+struct Row {
+  float2 m, w, e;
+};
+template <bool SIDES>
+__device__ __forceinline__ Row load_row(const float *p) {
+  Row v;
+  v.m = *reinterpret_cast<const float2 *>(p);
+  if (SIDES) {
+    v.w = make_float2(p[-1], v.m.x);
+    v.e = make_float2(v.m.y, p[2]);
+  }
+  return v;
 }
 
-__global__ void __launch_bounds__(NT_TILE) k_relax_tile(RelaxCoef r, const float *__restrict__ u,
-                                                        const float *__restrict__ gf, const float *__restrict__ phi,
-                                                        float *__restrict__ u_out) {
-  __shared__ float pl[3][3][HY][HX];          // [slot][component][y][x]
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
-  const int kb = blockIdx.z * KZ, ke = min(kb + KZ, r.nz);
-  const int i = i0 + tx, j = j0 + ty;
-  const bool live = i < r.nx && j < r.ny;
-  const int plane = r.ny * r.nx, cstride = r.nz * plane;
-  const int own = j * r.nx + i;
-  // the halo entries this thread stages, fixed for the whole march
-  int base[NQ], comp[NQ];
+template <bool STEP>
+__device__ __forceinline__ void read_plane(const RelaxCoef &r, const float *p, PlaneTerms &t) {
+  float2 xs[3], ys[3], cross[2];
 #pragma unroll
-  for (int e = 0; e < NQ; ++e) {
-    const int q = threadIdx.x + NT_TILE * e;
-    comp[e] = -1;
-    base[e] = 0;
-    if (q < PLANE) {
-      const int c = q / (HY * HX), rem = q - c * HY * HX;
-      const int hy = rem / HX, hx = rem - hy * HX;
-      comp[e] = c;
-      base[e] = c * cstride + mod(j0 + hy - 1, r.ny) * r.nx + mod(i0 + hx - 1, r.nx);
+  for (int c = 0; c < 3; ++c) {
+    const Row m = load_row<true>(p + c * CS);
+    const Row d = c < 2 ? load_row<STEP>(p + c * CS - LD) : load_row<false>(p + c * CS - LD);
+    const Row n = c < 2 ? load_row<STEP>(p + c * CS + LD) : load_row<false>(p + c * CS + LD);
+    t.c[c] = m.m;
+    if (STEP) {
+      xs[c] = add2(sub2(m.e, m.m), sub2(m.w, m.m));
+      ys[c] = add2(sub2(n.m, m.m), sub2(d.m, m.m));
+      if (c < 2) cross[c] = sub2(add2(n.e, d.w), add2(d.e, n.w));
+    }
+    if (c == 0) {
+      t.ax = sub2(m.e, m.w);
+      if (!STEP) t.in[1] = sub2(n.m, d.m);
+    } else if (c == 1) {
+      t.by = sub2(n.m, d.m);
+      if (!STEP) t.in[0] = sub2(m.e, m.w);
+    } else {
+      t.az = sub2(m.e, m.w);
+      t.bz = sub2(n.m, d.m);
     }
   }
-  int sb = 0, sm = 1, sa = 2;                 // slots of the layers below, at, above
-  float v[NQ];
-  fetch_plane(r, u, phi, base, comp, kb - 1, plane, v);
-  store_plane(v, comp, &pl[sb][0][0][0]);
-  fetch_plane(r, u, phi, base, comp, kb, plane, v);
-  store_plane(v, comp, &pl[sm][0][0][0]);
-  fetch_plane(r, u, phi, base, comp, kb + 1, plane, v);
-  store_plane(v, comp, &pl[sa][0][0][0]);
-  __syncthreads();
-  const int x = tx + 1, y = ty + 1;
-  for (int k = kb; k < ke; ++k) {
-    const bool more = k + 1 < ke;
-    if (more) fetch_plane(r, u, phi, base, comp, k + 2, plane, v);     // in flight during this layer
-    if (live) {
-      float (*B)[HY][HX] = pl[sb];
-      float (*C)[HY][HX] = pl[sm];
-      float (*A)[HY][HX] = pl[sa];
-      const int o = k * plane + own;
-      float out[3];
+  if (STEP) {                                      // d2u_y/dxdy into x, d2u_x/dxdy into y
+    t.in[0] = fma2(r.lap2[0][0], xs[0], fma2(r.lap2[0][1], ys[0], __fmul2_rn(r.mix2[0][1], cross[1])));
+    t.in[1] = fma2(r.lap2[1][0], xs[1], fma2(r.lap2[1][1], ys[1], __fmul2_rn(r.mix2[1][0], cross[0])));
+    t.in[2] = fma2(r.lap2[2][0], xs[2], __fmul2_rn(r.lap2[2][1], ys[2]));
+  }
+}
+
+// STEP: one explicit step, out[3] = u + dt (navier(u) + f), gin[3] = dt f.  Otherwise the
+// total stress, out[6] = gin[6] + lambda div u delta + mu (du_a/db + du_b/da).
+template <bool STEP, bool FULL>
+__global__ void __launch_bounds__(NTM, 2)
+k_relax_march(RelaxCoef r, const float *__restrict__ u, const float *gin, const float *__restrict__ phi, float *out,
+              int kz, int vec) {
+  constexpr int NC = STEP ? 3 : 6;
+  constexpr int SLOT = slot_floats<NC>();
+  extern __shared__ __align__(16) float ring[];
+  const int tx = threadIdx.x % PX, ty = threadIdx.x / PX;
+  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, i = i0 + 2 * tx;
+  const int kb = blockIdx.z * kz, ke = min(kb + kz, r.nz);
+  const bool live = FULL || (i < r.nx && j0 + ty < r.ny), second = FULL || i + 1 < r.nx;
+  const int plane = r.ny * r.nx, cstride = r.nz * plane, own = (j0 + ty) * r.nx + i;
+  const Stage st = make_stage(r, i0, j0);
+  const int mine = (ty + 1) * LD + X0 + 2 * tx, own_in = PLANE + 2 * threadIdx.x;
+  // one copy group, into slot q: plane k and the cells' inputs of layer k - 1 (nothing past
+  // the plane above the chunk)
+  auto start = [&](int k, int q) {
+    if (k <= ke) {
+      start_plane<FULL>(r, u, phi, st, i0, j0, k, vec, ring + q * SLOT);
+      if (live && k > kb) {
+        float *dst = ring + q * SLOT + own_in;
+        const int o = own + (k - 1) * plane;
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+          const float *src = gin + (o + c * cstride);
+          if constexpr (FULL) {
+            cp_async8f(dst + 2 * NTM * c, src);
+          } else {
+            cp_async4(dst + 2 * NTM * c, src);
+            if (second) cp_async4(dst + 2 * NTM * c + 1, src + 1);
+          }
+        }
+      }
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  PlaneTerms t[3];
+  int sq = 2;                                      // slot of plane k + 1
+  // layer k with the terms of the planes k - 1, k, k + 1 in t[P], t[P + 1], t[P + 2] (mod 3)
+  auto layer = [&](int k, auto P) {
+    constexpr int A = decltype(P)::value, B = (A + 1) % 3, D = (A + 2) % 3;
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 2) : "memory");      // plane k + 1 has landed
+    __syncthreads();                               // ... for every thread; planes up to k are read
+    start(k + RING, sq == 0 ? RING - 1 : sq - 1);
+    const float *slot = ring + sq * SLOT;
+    sq = sq == RING - 1 ? 0 : sq + 1;
+    read_plane<STEP>(r, slot + mine, t[D]);
+    float2 g[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) g[c] = *reinterpret_cast<const float2 *>(slot + own_in + 2 * NTM * c);
+    const PlaneTerms &lo = t[A], &mi = t[B], &up = t[D];
+    float2 v[NC];
+    if (STEP) {
+      const float2 mz[3] = {fma2(r.mix2[0][2], sub2(up.az, lo.az), mi.in[0]), fma2(r.mix2[1][2], sub2(up.bz, lo.bz), mi.in[1]),
+                            fma2(r.mix2[2][0], sub2(up.ax, lo.ax), fma2(r.mix2[2][1], sub2(up.by, lo.by), mi.in[2]))};
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        const float c0 = C[a][y][x];
-        float w = __ldg(gf + a * cstride + o);
-        w = fmaf(r.lap[a][0], (C[a][y][x + 1] - c0) + (C[a][y][x - 1] - c0), w);
-        w = fmaf(r.lap[a][1], (C[a][y + 1][x] - c0) + (C[a][y - 1][x] - c0), w);
-        w = fmaf(r.lap[a][2], (A[a][y][x] - c0) + (B[a][y][x] - c0), w);
-        out[a] = c0 + w;
+        const float2 c0 = mi.c[a];
+        const float2 w = fma2(r.lap2[a][2], add2(sub2(up.c[a], c0), sub2(lo.c[a], c0)), g[a]);
+        v[a] = add2(c0, add2(w, mz[a]));
       }
-      // 4-point crosses: d2u_y/dxdy, d2u_z/dxdz into x; d2u_x/dxdy, d2u_z/dydz into y;
-      // d2u_x/dxdz, d2u_y/dydz into z
-      const float uy_xy = (C[1][y + 1][x + 1] + C[1][y - 1][x - 1]) - (C[1][y - 1][x + 1] + C[1][y + 1][x - 1]);
-      const float ux_xy = (C[0][y + 1][x + 1] + C[0][y - 1][x - 1]) - (C[0][y - 1][x + 1] + C[0][y + 1][x - 1]);
-      const float uz_xz = (A[2][y][x + 1] + B[2][y][x - 1]) - (B[2][y][x + 1] + A[2][y][x - 1]);
-      const float ux_xz = (A[0][y][x + 1] + B[0][y][x - 1]) - (B[0][y][x + 1] + A[0][y][x - 1]);
-      const float uz_yz = (A[2][y + 1][x] + B[2][y - 1][x]) - (B[2][y + 1][x] + A[2][y - 1][x]);
-      const float uy_yz = (A[1][y + 1][x] + B[1][y - 1][x]) - (B[1][y + 1][x] + A[1][y - 1][x]);
-      out[0] += r.mix[0][1] * uy_xy + r.mix[0][2] * uz_xz;
-      out[1] += r.mix[1][0] * ux_xy + r.mix[1][2] * uz_yz;
-      out[2] += r.mix[2][0] * ux_xz + r.mix[2][1] * uy_yz;
+    } else {
+      const float2 hx = make_float2(r.inv2h[0], r.inv2h[0]), hy = make_float2(r.inv2h[1], r.inv2h[1]);
+      const float2 hz = make_float2(r.inv2h[2], r.inv2h[2]), mu = make_float2(r.mu, r.mu), mu2 = make_float2(2.f * r.mu, 2.f * r.mu);
+      const float2 xx = __fmul2_rn(mi.ax, hx), yy = __fmul2_rn(mi.by, hy), zz = __fmul2_rn(sub2(up.c[2], lo.c[2]), hz);
+      const float2 xy = fma2(mi.in[1], hy, __fmul2_rn(mi.in[0], hx));
+      const float2 xz = fma2(sub2(up.c[0], lo.c[0]), hz, __fmul2_rn(mi.az, hx));
+      const float2 yz = fma2(sub2(up.c[1], lo.c[1]), hz, __fmul2_rn(mi.bz, hy));
+      const float2 ld = __fmul2_rn(make_float2(r.lam, r.lam), add2(add2(xx, yy), zz));
+      const float2 e[6] = {fma2(mu2, xx, ld), fma2(mu2, yy, ld), fma2(mu2, zz, ld), __fmul2_rn(mu, xy), __fmul2_rn(mu, xz), __fmul2_rn(mu, yz)};
 #pragma unroll
-      for (int a = 0; a < 3; ++a) u_out[a * cstride + o] = out[a];
+      for (int c = 0; c < NC; ++c) v[c] = add2(g[c], e[c]);
     }
-    if (more) {
-      __syncthreads();                        // every thread is done with the plane below
-      const int t = sb;
-      sb = sm;
-      sm = sa;
-      sa = t;
-      store_plane(v, comp, &pl[sa][0][0][0]);
-      __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      float *p = out + (own + k * plane + c * cstride);
+      if constexpr (FULL) {
+        *reinterpret_cast<float2 *>(p) = v[c];
+      } else if (live) {
+        p[0] = v[c].x;
+        if (second) p[1] = v[c].y;
+      }
     }
-  }
-}
-
-// sigma_tot = sigma^dis + lambda div u delta + mu (du_a/db + du_b/da).
-__global__ void k_relax_stress(RelaxCoef r, const float *__restrict__ u, const float *__restrict__ phi,
-                               const float *__restrict__ sig, float *__restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y, k = blockIdx.z;
-  if (i >= r.nx || j >= r.ny) return;
-  float g[3][3];   // g[a][b] = du_a / db
+  };
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    g[a][0] = (uext(r, u, phi, a, i + 1, j, k) - uext(r, u, phi, a, i - 1, j, k)) * r.inv2h[0];
-    g[a][1] = (uext(r, u, phi, a, i, j + 1, k) - uext(r, u, phi, a, i, j - 1, k)) * r.inv2h[1];
-    g[a][2] = (uext(r, u, phi, a, i, j, k + 1) - uext(r, u, phi, a, i, j, k - 1)) * r.inv2h[2];
+  for (int q = 0; q < RING; ++q) start(kb - 1 + q, q);
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 2) : "memory");
+  __syncthreads();
+  read_plane<STEP>(r, ring + mine, t[0]);
+  read_plane<STEP>(r, ring + SLOT + mine, t[1]);
+  __syncthreads();                                 // slot 0 is read
+  start(kb - 1 + RING, 0);
+  using I0 = std::integral_constant<int, 0>;
+  using I1 = std::integral_constant<int, 1>;
+  using I2 = std::integral_constant<int, 2>;
+  for (int k = kb; k < ke; k += 3) {
+    layer(k, I0{});
+    if (k + 1 < ke) layer(k + 1, I1{});
+    if (k + 2 < ke) layer(k + 2, I2{});
   }
-  const float ld = r.lam * (g[0][0] + g[1][1] + g[2][2]);
-  const float s[6] = {ld + 2.f * r.mu * g[0][0], ld + 2.f * r.mu * g[1][1], ld + 2.f * r.mu * g[2][2],
-                      r.mu * (g[0][1] + g[1][0]), r.mu * (g[0][2] + g[2][0]), r.mu * (g[1][2] + g[2][1])};
-#pragma unroll
-  for (int c = 0; c < 6; ++c) out[cidx(r, c, k, j, i)] = __ldg(sig + cidx(r, c, k, j, i)) + s[c];
 }
 
 RelaxCoef relax_coef(const dds_ctx *ctx, double *dt_out) {
@@ -266,6 +409,8 @@ RelaxCoef relax_coef(const dds_ctx *ctx, double *dt_out) {
     for (int b = 0; b < 3; ++b) {
       r.lap[a][b] = (float)(dt * (a == b ? A : B) / (h[b] * h[b]));
       r.mix[a][b] = a == b ? 0.f : (float)(dt * (A - B) / (4.0 * h[a] * h[b]));
+      r.lap2[a][b] = make_float2(r.lap[a][b], r.lap[a][b]);
+      r.mix2[a][b] = make_float2(r.mix[a][b], r.mix[a][b]);
     }
     r.inv2h[a] = (float)(1.0 / (2.0 * h[a]));
   }
@@ -279,6 +424,32 @@ RelaxCoef relax_coef(const dds_ctx *ctx, double *dt_out) {
   r.dt = (float)dt;
   if (dt_out) *dt_out = dt;
   return r;
+}
+
+template <bool STEP>
+cudaError_t launch_march(const RelaxCoef &r, const float *u, const float *in, const float *phi, float *out,
+                         cudaStream_t s) {
+  // Layers per chunk: 16, or 8 or 4 where that would leave CTA slots (two per SM) idle.
+  // Longer chunks restart the march less often, but leave an emptier last wave (step on
+  // 256x256x128: 8 / 16 / 32 / 64 layers 82 / 77 / 82 / 81 us; 512x512x16: 8 / 16 layers
+  // 49 / 51 us; 100x90x40: 4 / 8 / 16 layers
+  // 11.9 / 12.3 / 20 us).
+  int dev = 0, sms = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (err != cudaSuccess) return err;
+  const long tiles = (long)((r.nx + TX - 1) / TX) * ((r.ny + TY - 1) / TY);
+  const int kz = tiles * ((r.nz + 15) / 16) >= 4 * sms ? 16 : (tiles * ((r.nz + 7) / 8) >= 2 * sms ? 8 : 4);
+  const dim3 grid((unsigned)((r.nx + TX - 1) / TX), (unsigned)((r.ny + TY - 1) / TY), (unsigned)((r.nz + kz - 1) / kz));
+  const int vec = r.nx % 4 == 0 && ((uintptr_t)u & 15) == 0;
+  const bool full = vec && r.nx % TX == 0 && r.ny % TY == 0 && (((uintptr_t)in | (uintptr_t)out) & 7) == 0;
+  const size_t smem = sizeof(float) * RING * slot_floats<STEP ? 3 : 6>();
+  auto kernel = full ? k_relax_march<STEP, true> : k_relax_march<STEP, false>;
+  err = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  if (err == cudaSuccess) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  kernel<<<grid, NTM, smem, s>>>(r, u, in, phi, out, kz, vec);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -309,16 +480,11 @@ int enqueue_relax(dds_ctx *ctx, const float *sig, float *u, int n_steps, float *
     a = tmp;
     b = u;
   }
-  const dim3 tgrid((unsigned)((r.nx + TX - 1) / TX), (unsigned)((r.ny + TY - 1) / TY), (unsigned)((r.nz + KZ - 1) / KZ));
   for (int t = 0; t < n_steps && err == cudaSuccess; ++t) {
-    k_relax_tile<<<tgrid, NT_TILE, 0, s>>>(r, a, gf, phi, b);
-    err = cudaGetLastError();
+    err = launch_march<true>(r, a, gf, phi, b, s);
     std::swap(a, b);
   }
-  if (err == cudaSuccess && sig_tot) {
-    k_relax_stress<<<grid, blk, 0, s>>>(r, u, phi, sig, sig_tot);
-    err = cudaGetLastError();
-  }
+  if (err == cudaSuccess && sig_tot) err = launch_march<false>(r, u, sig, phi, sig_tot, s);
   if (err != cudaSuccess) return fail(ctx, DDS_ERR_CUDA, "relax: kernel launch failed: %s", cudaGetErrorString(err));
   return DDS_OK;
 }
