@@ -63,7 +63,8 @@ enum {
   DDS_OPT_Z_LANES = 2,     /* schedule of the fused z pass: 0 = automatic (default);
                               -1 = shared-memory tiles; -2 = three-stage register kernel
                               (padded z size 128 or 256, <= 6 combined fields; the
-                              automatic choice there); 1, 2, 4, 8 = register-only kernel
+                              automatic choice there, and for padded z 512 up to 5 fields
+                              and 32 and 64 with 5 or 6); 1, 2, 4, 8 = register-only kernel
                               with that many lanes per (kx, ky) column (needs padded
                               z size <= 64 and <= 4 combined fields).  Same result up to
                               rounding; a tuning knob.  A schedule the grid cannot take

@@ -262,11 +262,17 @@ int make_plan(dds_ctx *ctx) {
     if (ctx->z_lanes > 0)
       return fail(ctx, DDS_ERR_UNSUPPORTED, "z pass: %d lanes per column not available for pz %d", G, sh.pz);
   }
-  // three-stage register z pass: padded z 128 or 256, at most 6 fields (default there)
+  // three-stage register z pass: padded z 128 or 256, at most 6 fields (on request, and the
+  // default there); by default also padded z 512 up to 5 fields (more than that has no
+  // schedule there), and 32 and 64 where more than four fields rule out the register-only pass: against shared-memory tiles, z pass of 90x77x200 (three
+  // fields) 0.81 -> 0.43 ms, of 250x241x29 (five fields, half the spectra) 0.37 -> 0.20 ms
   const int fw = zfour_width(sh.pz);
-  const bool four_ok = (sh.pz == 128 || sh.pz == 256) && sh.fe <= 6 && sh.M % fw == 0 && sh.py % fw == 0;
-  if (ctx->z_lanes == -2 || (ctx->z_lanes == 0 && ctx->z_wz == 0 && four_ok)) {
-    if (!four_ok)
+  const bool fits = sh.fe <= 6 && sh.M % fw == 0 && sh.py % fw == 0;
+  const bool four_ok = (sh.pz == 128 || sh.pz == 256) && fits;
+  const bool four_auto =
+      four_ok || (fits && (sh.pz == 512 ? sh.fe <= 5 : (sh.fe > 4 && (sh.pz == 32 || sh.pz == 64))));
+  if (ctx->z_lanes == -2 || (ctx->z_lanes == 0 && ctx->z_wz == 0 && four_auto)) {
+    if (ctx->z_lanes == -2 && !four_ok)
       return fail(ctx, DDS_ERR_UNSUPPORTED, "z pass: the three-stage kernel needs pz 128 or 256 and <= 6 fields "
                   "(pz %d, %d fields)", sh.pz, sh.fe);
     sh.zfour = 1;
@@ -559,9 +565,7 @@ int dds_autotune(dds_ctx *ctx, void *cuda_stream, float *best_ms) {
       if (base.pz % G == 0 && (E == 8 || E == 16) && base.M >= 32 / G) cand.push_back({G, 0});
     }
   }
-  if ((base.pz == 128 || base.pz == 256) && base.fe <= 6 && base.M % zfour_width(base.pz) == 0 &&
-      base.py % zfour_width(base.pz) == 0)
-    cand.push_back({-2, 0});
+  if (base.zfour) cand.push_back({0, 0});        // the automatic choice here
   for (int W : {4, 8, 16, 32, 64}) {
     if (W > base.M || base.py % W != 0 || (W * base.pz > 2048 && W > 8)) continue;
     const size_t fe = (size_t)std::max(base.fe, 1);
@@ -589,7 +593,7 @@ int dds_autotune(dds_ctx *ctx, void *cuda_stream, float *best_ms) {
     rc = make_plan(ctx);
     if (rc != DDS_OK) break;
     if (ctx->shape.zreg_g != (cand[i].first > 0 ? cand[i].first : 0)) continue;   // planner declined
-    if (ctx->shape.zfour != (cand[i].first == -2 ? 1 : 0)) continue;
+    if (ctx->shape.zfour != (cand[i].first == 0 ? 1 : 0)) continue;
     rc = alloc_buffers(ctx);
     if (rc != DDS_OK) break;
     const size_t vbytes = ctx->spectra_fp16 ? 2 : sizeof(float);

@@ -547,9 +547,9 @@ __global__ void k_extract(const double *spec, int fold, int M, int py, int pz, i
 }
 
 // Imaginary part of the spectrum of component c of field e, scaled, into the layout
-// the three-stage z pass reads (pz = 8 R1, tiles of W = wz columns): per stored tile s
+// the three-stage z pass reads (pz = R1 R2, tiles of W = wz columns): per stored tile s
 // and component c, 16-byte chunks [j][thread t = k1 W + w], the value of
-// (e, kz = k1 + R1 k2) at position (8 e + k2) % V of chunk j = (8 e + k2) / V, V values
+// (e, kz = k1 + R1 k2) at position (R2 e + k2) % V of chunk j = (R2 e + k2) / V, V values
 // per chunk.  Stored tiles: the main tiles (ky, kx tile) row by row -- all of them, or
 // those with ky <= py/2 when every field has the x-mirror parity (ZSym::xall) -- then
 // the Nyquist tiles (kx = M).
@@ -557,12 +557,12 @@ template <typename OT>
 __global__ void k_extract_four(const double *spec, int fold, Shape sh, int e, int c, double scale,
                                const unsigned long long *amax, OT *kspec) {
   constexpr int V = 16 / (int)sizeof(OT);
-  const int W = sh.wz, R1 = sh.pz / 8, M = sh.M, py = sh.py, fe = sh.fe;
+  const int W = sh.wz, R2 = zfour_r2(sh.pz), R1 = sh.pz / R2, M = sh.M, py = sh.py, fe = sh.fe;
   const long per_tile = (long)sh.pz * W;
   const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (idx >= zf_stored_tiles(sh) * per_tile) return;
   const long s = idx / per_tile;
-  const int r = (int)(idx - s * per_tile), t = r / 8, k2 = r % 8, k1 = t / W, w = t % W, q = 8 * e + k2;
+  const int r = (int)(idx - s * per_tile), t = r / R2, k2 = r % R2, k1 = t / W, w = t % W, q = R2 * e + k2;
   const long ktiles = M / W;
   const long main_tiles = (long)(sh.zs.xall ? py / 2 + 1 : py) * ktiles;
   int kx, ky;

@@ -48,14 +48,15 @@ struct Shape {
   int fin, fe;        // input families, effective fields
   int wz;             // columns per tile of the fused z pass (shared-memory variant)
   int zreg_g;         // > 0: register-only z pass, pz = 16 * zreg_g, zreg_g lanes per column
-  int zfour;          // 1: three-stage register z pass (pz 128 or 256, wz = zfour_width(pz))
+  int zfour;          // 1: three-stage register z pass (wz = zfour_width(pz))
   int nb;             // density sets evaluated together (batch); fields are [b][e], outputs [b][c]
   ZSym zs;            // zfour: stored-spectrum symmetries and layout
   int yxf;            // > 0: fused inverse y + x pass, one cluster of yxf CTAs per plane
 };
 
-// Columns per tile of the three-stage z pass (Shape::zfour) for padded z size pz.
-__host__ __device__ constexpr int zfour_width(int pz) { return pz >= 256 ? 8 : 16; }
+// Three-stage z pass (Shape::zfour) for padded z size pz = R1 R2: columns per tile, and R2.
+__host__ __device__ constexpr int zfour_width(int pz) { return pz >= 512 ? 4 : pz >= 256 ? 8 : pz >= 128 ? 16 : 32; }
+__host__ __device__ constexpr int zfour_r2(int pz) { return pz >= 512 ? 16 : 8; }
 
 // Tiles of the three-stage z pass whose kernel spectra are stored: the main tiles
 // (all ky, or ky <= py/2 under xall), then the py / W Nyquist-column tiles.

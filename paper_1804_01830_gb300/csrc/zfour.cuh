@@ -1,20 +1,21 @@
-// Fused z pass for padded z sizes 128 and 256 (PZ = 8 R1), in three register stages
-// of the four-step factorisation: forward n = n2 + 8 n1, k = k1 + R1 k2; inverse
-// k = k1 + R1 k2, n = a + 8 b.  A CTA takes W adjacent columns (16 for PZ 128: rows of
-// 128 bytes; 8 for PZ 256, so that two CTAs fit an SM) with R1 W threads:
-//   stage 1  thread (field e, n2, column w) loads rows n2 + 8 n1 < nz straight from
+// Fused z pass for padded z sizes 128, 256 and 512, and 32 and 64 with more than four
+// fields, in three register stages of the four-step factorisation PZ = R1 R2 (R2 = 8, or
+// 16 for PZ 512): forward n = n2 + R2 n1, k = k1 + R1 k2; inverse k = k1 + R1 k2,
+// n = a + R2 b.  A CTA takes W adjacent columns (tiles of 2048 points, so that two CTAs fit
+// an SM; 1024 for PZ 32) with R1 W threads:
+//   stage 1  thread (field e, n2, column w) loads rows n2 + R2 n1 < nz straight from
 //            global memory (row segments of W complex values), runs the R1-point DFT of the
 //            half-zero input (two R1/2-point DFTs), twiddles by W_PZ^(n2 k1) and
 //            writes T[e][k1][n2][w];
-//   stage 2  thread (k1, w) reads its 8 values of every field, runs the 8-point DFTs
+//   stage 2  thread (k1, w) reads its R2 values of every field, runs the R2-point DFTs
 //            and keeps rho^_e(k1 + R1 k2) of all fields in registers; for each
 //            component it loads its kernel spectra straight from global memory (laid
 //            out per thread in 16-byte chunks), contracts (Eq. 10 in Fourier space),
-//            runs the inverse 8-point DFT over k2, twiddles by conj W_PZ^(a k1) and
+//            runs the inverse R2-point DFT over k2, twiddles by conj W_PZ^(a k1) and
 //            writes Y[c][a][k1][w] into the space of T;
 //   stage 3  thread (c, a, w) reads the R1 values of k1, runs the inverse R1-point DFT
-//            for the outputs b < R1/2 only (rows a + 8 b < nz <= PZ/2) and stores them.
-// Shared memory is written and read once per stage; row strides of 9 W values (T) and
+//            for the outputs b < R1/2 only (rows a + R2 b < nz <= PZ/2) and stores them.
+// Shared memory is written and read once per stage; row strides of (R2 + 1) W values (T) and
 // (R1 + 1) W values (Y) keep every stage's half-warp accesses free of bank conflicts.
 //
 // Kernel spectra of fields with the x-mirror parity (ZSym) are stored for ky <= py/2
@@ -32,10 +33,12 @@ namespace zp {
 
 template <int PZ> struct ZF {
   static constexpr int W = zfour_width(PZ);   // columns per tile
-  static constexpr int R2 = 8, R1 = PZ / 8, NT = R1 * W;
-  static constexpr int SK = (R2 + 1) * W;     // T row (e, k1): 8 n2 x W columns + W
+  static constexpr int R2 = zfour_r2(PZ), R1 = PZ / R2, NT = R1 * W;
+  static constexpr int SK = (R2 + 1) * W;     // T row (e, k1): R2 n2 x W columns + W
   static constexpr int SY = (R1 + 1) * W;     // Y row (c, a): R1 k1 x W columns + W
-  static_assert(R1 == 16 || R1 == 32, "padded z size 128 or 256");
+  // items of stage 1 whose rows a thread requests before it transforms any
+  static constexpr int IPR = R1 >= 16 ? 2 : R1 == 8 ? 5 : 8;
+  static_assert(R1 * R2 == PZ && R1 >= 4 && NT <= 256, "padded z size 32 to 512");
 };
 
 // shared memory of the kernel, in float2 values: T, or Y in the same space ...
@@ -62,36 +65,38 @@ __device__ __forceinline__ void zf_tile_of(int L, int py, int ktiles, int *ky, i
   *ky = ((L - 2 * ktiles) & 1) ? py - ky1 : ky1;
 }
 
-// The kernel-spectrum values (e, k2 = 0..7) of fields e = e0 .. e0 + FE - 1 of one
+// The kernel-spectrum values (e, k2 < R2) of fields e = e0 .. e0 + FE - 1 of one
 // component for the calling thread, held raw in registers (FP32, or FP16 converted and
 // scaled at use).  Layout of one (tile, component): 16-byte chunks [j][thread], value
-// (e, k2) in chunk j = (8 e + k2) / (values per chunk).
-template <typename GT, int FE> struct ZRaw;
-template <int FE> struct ZRaw<float, FE> {
-  float4 v[FE][2];
+// (e, k2) in chunk j = (R2 e + k2) / (values per chunk).
+template <typename GT, int FE, int R2> struct ZRaw;
+template <int FE, int R2> struct ZRaw<float, FE, R2> {
+  float4 v[FE][R2 / 4];
   __device__ __forceinline__ void load(const float *kc, int e0, int t, int nthreads) {
     const float4 *p = reinterpret_cast<const float4 *>(kc);
 #pragma unroll
-    for (int e = 0; e < FE; ++e) {
-      v[e][0] = __ldg(p + (long)(2 * (e0 + e)) * nthreads + t);
-      v[e][1] = __ldg(p + (long)(2 * (e0 + e) + 1) * nthreads + t);
-    }
+    for (int e = 0; e < FE; ++e)
+#pragma unroll
+      for (int q = 0; q < R2 / 4; ++q) v[e][q] = __ldg(p + (R2 / 4 * (e0 + e) + q) * nthreads + t);
   }
   __device__ __forceinline__ float get(int e, int k2, float) const {
     const float4 q = v[e][k2 / 4];
     return (k2 % 4 == 0) ? q.x : (k2 % 4 == 1) ? q.y : (k2 % 4 == 2) ? q.z : q.w;
   }
 };
-template <int FE> struct ZRaw<__half, FE> {
-  uint4 v[FE];
+template <int FE, int R2> struct ZRaw<__half, FE, R2> {
+  uint4 v[FE][R2 / 8];
   __device__ __forceinline__ void load(const __half *kc, int e0, int t, int nthreads) {
     const uint4 *p = reinterpret_cast<const uint4 *>(kc);
 #pragma unroll
-    for (int e = 0; e < FE; ++e) v[e] = __ldg(p + (long)(e0 + e) * nthreads + t);
+    for (int e = 0; e < FE; ++e)
+#pragma unroll
+      for (int q = 0; q < R2 / 8; ++q) v[e][q] = __ldg(p + (R2 / 8 * (e0 + e) + q) * nthreads + t);
   }
   __device__ __forceinline__ float get(int e, int k2, float s) const {
-    const uint4 q = v[e];
-    const unsigned w = (k2 / 2 == 0) ? q.x : (k2 / 2 == 1) ? q.y : (k2 / 2 == 2) ? q.z : q.w;
+    const uint4 q = v[e][k2 / 8];
+    const int h = k2 % 8 / 2;
+    const unsigned w = h == 0 ? q.x : h == 1 ? q.y : h == 2 ? q.z : q.w;
     const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w));
     return ((k2 % 2) ? f.y : f.x) * s;
   }
@@ -103,7 +108,7 @@ __device__ __forceinline__ void prefetch_l2_bulk(const void *p, unsigned bytes) 
 }
 
 template <int PZ, int FE, typename GT>
-__global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
+__global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
     k_zfour(Shape sh, const float2 *in_main, const float2 *in_nyq, const GT *kspec, const float *kscale,
             float2 *out_main, float2 *out_nyq, const float2 *tw) {
   constexpr int R1 = ZF<PZ>::R1, R2 = ZF<PZ>::R2, W = ZF<PZ>::W, NT = ZF<PZ>::NT;
@@ -142,7 +147,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
       prefetch_l2_bulk(reinterpret_cast<const char *>(ks) + tid * CH, min(CH, BYTES - tid * CH));
   };
 
-  // stage 1: forward R1-point DFTs over n1 of the rows n2 + 8 n1 (n1 < R1/2 non-zero);
+  // stage 1: forward R1-point DFTs over n1 of the rows n2 + R2 n1 (n1 < R1/2 non-zero);
   // a negated-frequency tile transforms -s_b conj(rho) (s_b folds the spectra's sign)
   constexpr int NI = FE * R2 * W;              // items (field, n2, column)
   // element (e, z, w) of the tile's rows: src[e se + z sz + w sw1].  One pointer for both
@@ -179,27 +184,45 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
       T[(2 * j + 1) * SK] = cmul_tw<false>(od[j], twP[n2 * (2 * j + 1)]);
     }
   };
-  // items in pairs of rounds: both items' rows are requested before either is transformed
-  // (five fields give 1.25 items per thread; GaN layer 1.11 -> 1.07 ms)
-  for (int item = tid; item < NI; item += 2 * NT) {
-    float2 a[H], b[H];
-    const bool two = item + NT < NI;
-    s1_load(item, a);
-    if (two) s1_load(item + NT, b);
-    // the rows first: requested ahead of them, the spectra delay them (GaN layer, with the
-    // single pointer: 1.04 -> 0.93 ms)
-    if (item == tid) prefetch_spectra();
-    s1_finish(item, a);
-    if (two) s1_finish(item + NT, b);
+  // the rows of IPR items are requested before any is transformed (in pairs: GaN layer 1.11
+  // -> 1.07 ms; padded z 64, five items per thread, all five instead of pairs: film of
+  // 250x241x29 0.232 -> 0.202 ms; three or four at padded z 128 measured slower than pairs).
+  // The rows go first: requested ahead of them, the spectra delay them (GaN layer, with the
+  // single pointer: 1.04 -> 0.93 ms).
+  constexpr int IPR = ZF<PZ>::IPR;
+  if constexpr (IPR == 2) {
+    for (int item = tid; item < NI; item += 2 * NT) {
+      float2 a[H], b[H];
+      const bool two = item + NT < NI;
+      s1_load(item, a);
+      if (two) s1_load(item + NT, b);
+      if (item == tid) prefetch_spectra();
+      s1_finish(item, a);
+      if (two) s1_finish(item + NT, b);
+    }
+  } else {
+    for (int item = tid; item < NI; item += IPR * NT) {
+      float2 a[IPR][H];
+      bool ok[IPR];
+#pragma unroll
+      for (int q = 0; q < IPR; ++q) {
+        ok[q] = q == 0 || item + q * NT < NI;
+        if (ok[q]) s1_load(item + q * NT, a[q]);
+      }
+      if (item == tid) prefetch_spectra();
+#pragma unroll
+      for (int q = 0; q < IPR; ++q)
+        if (ok[q]) s1_finish(item + q * NT, a[q]);
+    }
   }
   __syncthreads();
 
-  // stage 2: forward 8-point DFTs over n2, contraction, inverse 8-point DFTs over k2;
+  // stage 2: forward R2-point DFTs over n2, contraction, inverse R2-point DFTs over k2;
   // the spectra of the next component (of its first PF fields, as registers allow) load
   // while the current one is inverted and stored
   constexpr int PF = FE <= 4 ? FE : (FE == 5 ? 2 : 1);
   const int k1 = tid / W, w = tid - k1 * W;
-  ZRaw<GT, PF> gr;
+  ZRaw<GT, PF, R2> gr;
   gr.load(ks, 0, tid, NT);
   float2 f[FE][R2];
 #pragma unroll
@@ -216,7 +239,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
 #pragma unroll
     for (int k2 = 0; k2 < R2; ++k2) s[k2] = make_float2(0.f, 0.f);
     // this component's other fields load now, before the prefetched ones are used
-    ZRaw<GT, (FE > PF ? FE - PF : 1)> lt;
+    ZRaw<GT, (FE > PF ? FE - PF : 1), R2> lt;
     if constexpr (FE > PF) lt.load(kc, PF, tid, NT);
 #pragma unroll
     for (int e = 0; e < PF; ++e) {
@@ -231,7 +254,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, 512 / ZF<PZ>::NT)
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) s[k2] = cmadd_i(s[k2], lt.get(e - PF, k2, sc), f[e][k2]);
     }
-    dft_reg<R2, true>(s);                     // index a of n = a + 8 b
+    dft_reg<R2, true>(s);                     // index a of n = a + R2 b
     float2 *Y = zsm + (long)c * R2 * SY + k1 * W + w;
     Y[0] = s[0];
 #pragma unroll
@@ -284,18 +307,23 @@ cudaError_t launch_zfour(const Shape &sh, const float2 *im, const float2 *in, co
   return cudaGetLastError();
 }
 
-template <int PZ, typename GT>
+// FMIN, FMAX: the fewest and most fields the plan gives this padded z size.
+template <int PZ, int FMIN, int FMAX, typename GT>
 cudaError_t dispatch_zfour_fe(const Shape &sh, const float2 *im, const float2 *in, const GT *ks, const float *ksc,
                               float2 *om, float2 *on, const float2 *tw, cudaStream_t s) {
-  switch (sh.fe) {
-    case 1: return launch_zfour<PZ, 1, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    case 2: return launch_zfour<PZ, 2, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    case 3: return launch_zfour<PZ, 3, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    case 4: return launch_zfour<PZ, 4, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    case 5: return launch_zfour<PZ, 5, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    case 6: return launch_zfour<PZ, 6, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    default: return cudaErrorInvalidValue;
+  if (sh.fe == 5) return launch_zfour<PZ, 5, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+  if constexpr (FMAX == 6)
+    if (sh.fe == 6) return launch_zfour<PZ, 6, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+  if constexpr (FMIN == 1) {
+    switch (sh.fe) {
+      case 1: return launch_zfour<PZ, 1, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 2: return launch_zfour<PZ, 2, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 3: return launch_zfour<PZ, 3, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 4: return launch_zfour<PZ, 4, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      default: break;
+    }
   }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace zp

@@ -430,9 +430,14 @@ template <typename GT>
 cudaError_t dispatch_z_typed(const Shape &sh, const float2 *im, const float2 *in, const GT *ks, const float *ksc,
                              float2 *om, float2 *on, const float2 *tw, cudaStream_t s) {
   if (sh.zfour) {
-    if (sh.pz == 128) return dispatch_zfour_fe<128, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    if (sh.pz == 256) return dispatch_zfour_fe<256, GT>(sh, im, in, ks, ksc, om, on, tw, s);
-    return cudaErrorInvalidValue;
+    switch (sh.pz) {
+      case 32: return dispatch_zfour_fe<32, 5, 6, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 64: return dispatch_zfour_fe<64, 5, 6, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 128: return dispatch_zfour_fe<128, 1, 6, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 256: return dispatch_zfour_fe<256, 1, 6, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      case 512: return dispatch_zfour_fe<512, 1, 5, GT>(sh, im, in, ks, ksc, om, on, tw, s);
+      default: return cudaErrorInvalidValue;
+    }
   }
   if (sh.zreg_g > 0) {
     switch (sh.pz * 16 + sh.zreg_g) {   // (pz, lanes per column) -> E = pz / G registers
