@@ -51,6 +51,7 @@ struct Shape {
   int zfour;          // 1: three-stage register z pass (wz = zfour_width(pz))
   int nb;             // density sets evaluated together (batch); fields are [b][e], outputs [b][c]
   ZSym zs;            // zfour: stored-spectrum symmetries and layout
+  int early;          // launches may start before the kernel ahead of them has finished
   int yxf;            // > 0: fused inverse y + x pass, one cluster of yxf CTAs per plane
 };
 

@@ -37,8 +37,6 @@ __device__ int g_wait_status;
 
 namespace {
 
-constexpr int MAX_DEV = 64;
-
 // Per device: SM count and the address of g_wait_status (looked up once).
 struct DevInfo {
   int sms = 0;
@@ -65,16 +63,23 @@ cudaError_t dev_info(DevInfo *out) {
 }
 
 // Persistent grid: as many CTAs as fit on the device at once, at most one per tile.
-template <typename K>
-cudaError_t persistent_grid(K kernel, int threads, size_t smem, long tiles, const DevInfo &di, unsigned *grid) {
-  int per_sm = 0;
-  const cudaError_t err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+template <auto Kernel>
+cudaError_t persistent_grid(int threads, size_t smem, long tiles, const DevInfo &di, unsigned *grid) {
+  static std::atomic<int> resident[MAX_DEV];   // CTAs per SM (looked up once per device)
+  int dev = 0;
+  cudaError_t err = cudaGetDevice(&dev);
+  if (err == cudaSuccess) err = pass_attributes<Kernel, true>(dev, smem);
   if (err != cudaSuccess) return err;
-  const long g = std::max(1L, std::min(tiles, (long)std::max(per_sm, 1) * di.sms));
-  *grid = (unsigned)g;
+  int per_sm = resident[dev].load(std::memory_order_relaxed);
+  if (per_sm == 0) {
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem);
+    if (err != cudaSuccess) return err;
+    per_sm = std::max(per_sm, 1);
+    resident[dev].store(per_sm, std::memory_order_relaxed);
+  }
+  *grid = (unsigned)std::max(1L, std::min(tiles, (long)per_sm * di.sms));
   return cudaSuccess;
 }
-
 
 // ------------------------------------------------------------- y passes -----
 // Forward: rows y < ny in, all py rows out.  Inverse: all py rows in, y < ny out.
@@ -84,6 +89,8 @@ __global__ void __launch_bounds__(NT) k_ypass(Shape sh, int nf, const float2 *in
   constexpr int LD = W, PB = Plan<PY>::r0;
   extern __shared__ float2 smem[];
   float2 *buf = smem;
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x;
   const int M = sh.M, nz = sh.nz;
   const int rows_in = INV ? PY : sh.ny;
@@ -149,6 +156,8 @@ __global__ void __launch_bounds__(NT) k_ypass(Shape sh, int nf, const float2 *in
 
 // s = sqrt(sum / (nx ny)) for every (set, component, height).
 __global__ void k_stats_finish(const double *sums, long n, double inv_plane, float *s_out) {
+  pdl_trigger();
+  pdl_wait();
   const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (i < n) s_out[i] = (float)sqrt(sums[i] * inv_plane);
 }
@@ -161,10 +170,7 @@ cudaError_t launch_x_fwd_kind(const Shape &sh, const Collapse &col, const GroupL
   constexpr int LPB = xr::THREADS / (xr::FwdCfg<M>::R1 / 2);
   const long L = (long)sh.ny * sh.nz;
   dim3 grid((unsigned)((L + LPB - 1) / LPB), gl.n, sh.nb);
-  cudaError_t err = prep(xr::k_x_fwd_reg<M, BF16, DIRECT>, 0);
-  if (err != cudaSuccess) return err;
-  xr::k_x_fwd_reg<M, BF16, DIRECT><<<grid, xr::THREADS, 0, s>>>(sh, col, gl, rho, om, on, tw);
-  return cudaGetLastError();
+  return launch_pass<xr::k_x_fwd_reg<M, BF16, DIRECT>>(sh.early, grid, xr::THREADS, 0, s, sh, col, gl, rho, om, on, tw);
 }
 
 // Groups with one family and one field transform that family directly; the others
@@ -199,10 +205,7 @@ cudaError_t launch_y(const Shape &sh, int nf, const float2 *im, const float2 *in
   if (sh.py == sh.ny) {                   // periodic in y: no zero padding (py <= 512)
     if constexpr (PY <= 512) {
       const size_t smem = sizeof(float2) * yr::y_smem_all<PY, W, INV, true>();
-      cudaError_t err = prep(yr::k_ypass_st<PY, W, T, INV, true>, smem);
-      if (err != cudaSuccess) return err;
-      yr::k_ypass_st<PY, W, T, INV, true><<<(unsigned)tiles, T, smem, s>>>(sh, nf, im, in, om, on, tw);
-      return cudaGetLastError();
+      return launch_pass<yr::k_ypass_st<PY, W, T, INV, true>>(sh.early, (unsigned)tiles, T, smem, s, sh, nf, im, in, om, on, tw);
     }
     return cudaErrorInvalidValue;
   }
@@ -211,16 +214,10 @@ cudaError_t launch_y(const Shape &sh, int nf, const float2 *im, const float2 *in
     // disk 512x512x16: 0.137 ms, against 0.152 for the register stages on 4-column
     // tiles and 0.146 on 8-column tiles of 256 threads)
     const size_t smem = sizeof(float2) * tile_elems<PY, W, Plan<PY>::r0, W>();
-    cudaError_t err = prep(k_ypass<PY, W, T, INV>, smem);
-    if (err != cudaSuccess) return err;
-    k_ypass<PY, W, T, INV><<<(unsigned)tiles, T, smem, s>>>(sh, nf, im, in, om, on, tw);
-    return cudaGetLastError();
+    return launch_pass<k_ypass<PY, W, T, INV>>(sh.early, (unsigned)tiles, T, smem, s, sh, nf, im, in, om, on, tw);
   }
   const size_t smem = sizeof(float2) * yr::y_smem_all<PY, W, INV, false>();
-  cudaError_t err = prep(yr::k_ypass_st<PY, W, T, INV>, smem);
-  if (err != cudaSuccess) return err;
-  yr::k_ypass_st<PY, W, T, INV><<<(unsigned)tiles, T, smem, s>>>(sh, nf, im, in, om, on, tw);
-  return cudaGetLastError();
+  return launch_pass<yr::k_ypass_st<PY, W, T, INV, false>>(sh.early, (unsigned)tiles, T, smem, s, sh, nf, im, in, om, on, tw);
 }
 
 
@@ -235,13 +232,11 @@ cudaError_t launch_x_inv(const Shape &sh, const float2 *im, const float2 *in, fl
   const long L = 6L * sh.nb * sh.nz * sh.ny;
   DevInfo di;
   cudaError_t err = dev_info(&di);
-  if (err == cudaSuccess) err = prep(xr::k_x_inv_tma<M>, C::SMEM);
   unsigned grid = 0;
   if (err == cudaSuccess)
-    err = persistent_grid(xr::k_x_inv_tma<M>, xr::THREADS, C::SMEM, (L + C::LPB - 1) / C::LPB, di, &grid);
+    err = persistent_grid<xr::k_x_inv_tma<M>>(xr::THREADS, C::SMEM, (L + C::LPB - 1) / C::LPB, di, &grid);
   if (err != cudaSuccess) return err;
-  xr::k_x_inv_tma<M><<<grid, xr::THREADS, C::SMEM, s>>>(sh, im, in, sigma, tw, stats, di.status);
-  return cudaGetLastError();
+  return launch_pass<xr::k_x_inv_tma<M>>(sh.early, grid, xr::THREADS, C::SMEM, s, sh, im, in, sigma, tw, stats, di.status);
 }
 
 // Fused inverse y + x pass (yxpass.cuh): one cluster of Cfg::CL CTAs per output plane.
@@ -376,10 +371,13 @@ int enqueue_stress(dds_ctx *ctx, const void *rho, int rho_dtype, float *sigma, c
   Shape sh = ctx->shape;
   sh.nb = nb;
   if (sub) sh.fin = sub_fin;
+  // a captured chain keeps full dependencies: programmatic edges add 3 us to each replay
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t err = cudaStreamIsCapturing(s, &capture);
+  sh.early = err == cudaSuccess && capture == cudaStreamCaptureStatusNone;
   const Collapse &col = sub ? *sub : ctx->col;
   const float2 *tw = ctx->tw.f32;
   cudaEvent_t *ev = nullptr;
-  cudaError_t err = cudaSuccess;
   if (ctx->profiling) {
     const size_t need = 6 * (size_t)(ctx->prof_steps + 1);
     while (err == cudaSuccess && ctx->prof_events.size() < need) {
@@ -396,6 +394,7 @@ int enqueue_stress(dds_ctx *ctx, const void *rho, int rho_dtype, float *sigma, c
   auto mark = [&](int i) {
     if (ev && err == cudaSuccess) err = cudaEventRecord(ev[i], s);
   };
+  if (err == cudaSuccess && stats != nullptr) err = cudaMemsetAsync(stats, 0, sizeof(double) * 6 * nb * sh.nz, s);
   if (err == cudaSuccess) err = dispatch_x_fwd(sh, col, rho, rho_dtype == DDS_BF16, ctx->bufA, ctx->nyqA, tw, s);
   mark(1);
   if (err == cudaSuccess) err = dispatch_y<false>(sh, nb * sh.fe, ctx->bufA, ctx->nyqA, ctx->bufB, ctx->nyqB, tw, s);
@@ -406,14 +405,13 @@ int enqueue_stress(dds_ctx *ctx, const void *rho, int rho_dtype, float *sigma, c
   if (err == cudaSuccess && sh.yxf == 0)
     err = dispatch_y<true>(sh, 6 * nb, ctx->bufA, ctx->nyqA, ctx->bufB, ctx->nyqB, tw, s);
   mark(4);
-  if (err == cudaSuccess && stats != nullptr) err = cudaMemsetAsync(stats, 0, sizeof(double) * 6 * nb * sh.nz, s);
   if (err == cudaSuccess)
     err = sh.yxf > 0 ? dispatch_yx_inv(sh, ctx->bufA, ctx->nyqA, sigma, tw, s, stats)
                      : dispatch_x_inv(sh, ctx->bufB, ctx->nyqB, sigma, tw, s, stats);
   if (err == cudaSuccess && stats != nullptr) {
     const long n = 6L * nb * sh.nz;
-    k_stats_finish<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(stats, n, 1.0 / ((double)sh.nx * sh.ny), s_out);
-    err = cudaGetLastError();
+    err = launch_pass<k_stats_finish, false>(sh.early, (unsigned)((n + 255) / 256), 256, 0, s, stats, n, 1.0 / ((double)sh.nx * sh.ny),
+                                      s_out);
   }
   mark(5);
   if (err != cudaSuccess) return fail(ctx, DDS_ERR_CUDA, "stress: kernel launch failed: %s", cudaGetErrorString(err));
@@ -423,9 +421,12 @@ int enqueue_stress(dds_ctx *ctx, const void *rho, int rho_dtype, float *sigma, c
 // The five passes on caller-provided work buffers (used by dds_stress_noalloc).
 int enqueue_stress_buffers(dds_ctx *ctx, const void *rho, int rho_dtype, float *sigma, float2 *bufA, float2 *bufB,
                            float2 *nyqA, float2 *nyqB, cudaStream_t s) {
-  const Shape &sh = ctx->shape;
+  Shape sh = ctx->shape;
   const float2 *tw = ctx->tw.f32;
-  cudaError_t err = dispatch_x_fwd(sh, ctx->col, rho, rho_dtype == DDS_BF16, bufA, nyqA, tw, s);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t err = cudaStreamIsCapturing(s, &capture);
+  sh.early = err == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+  if (err == cudaSuccess) err = dispatch_x_fwd(sh, ctx->col, rho, rho_dtype == DDS_BF16, bufA, nyqA, tw, s);
   if (err == cudaSuccess) err = dispatch_y<false>(sh, sh.fe, bufA, nyqA, bufB, nyqB, tw, s);
   if (err == cudaSuccess) err = dispatch_z(sh, bufB, nyqB, ctx->kspec, ctx->kscale, bufA, nyqA, tw, s);
   if (sh.yxf > 0) {

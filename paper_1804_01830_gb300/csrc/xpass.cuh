@@ -99,10 +99,9 @@ k_x_inv_tma(Shape sh, const float2 *__restrict__ in_main, const float2 *__restri
   const long L = 6L * sh.nb * sh.nz * sh.ny;
   const long ntiles = (L + LPB - 1) / LPB;
   const long stride = gridDim.x;
-  for (int i = threadIdx.x; i < M; i += THREADS) {
-    stwM[i] = __ldg(tw + tw_offset(M) + i);
-    stwM[M + i] = __ldg(tw + tw_offset(2 * M) + i);
-  }
+  pdl_trigger();
+  stage_table<THREADS>(stwM, tw + tw_offset(M), M, threadIdx.x);
+  stage_table<THREADS>(stwM + M, tw + tw_offset(2 * M), M, threadIdx.x);
   const float2 *twM = stwM;
   const float2 *tw2 = stwM + M;
   const int nxh = (sh.nx + 1) >> 1;
@@ -120,6 +119,7 @@ k_x_inv_tma(Shape sh, const float2 *__restrict__ in_main, const float2 *__restri
     fence_mbar_init();
   }
   __syncthreads();
+  pdl_wait();
   // thread 0 only: copies issued and not yet waited for, and the barrier phase
   // (parity) each will complete; use j of slot j & 1 completes phase (j >> 1) & 1
   bool pending[2] = {false, false};
@@ -131,8 +131,9 @@ k_x_inv_tma(Shape sh, const float2 *__restrict__ in_main, const float2 *__restri
   float2 xm_next = make_float2(0.f, 0.f);
   {
     const long line = (long)blockIdx.x * LPB + lw;
-    if (t0 && blockIdx.x < ntiles && line < L) xm_next = in_nyq[nyq_index(sh, line)];
+    if (t0 && blockIdx.x < ntiles && line < L) xm_next = ld_cg(in_nyq + nyq_index(sh, line));
   }
+  cp_async_wait_all();                        // tables: visible to the CTA after the first tile's barrier
   bool ok = true;
   for (long i = 0;; ++i) {
     const long tile = blockIdx.x + i * stride;
@@ -145,7 +146,7 @@ k_x_inv_tma(Shape sh, const float2 *__restrict__ in_main, const float2 *__restri
     const float2 xm = xm_next;
     {
       const long nline = (tile + stride) * LPB + lw;
-      xm_next = (t0 && tile + stride < ntiles && nline < L) ? in_nyq[nyq_index(sh, nline)] : make_float2(0.f, 0.f);
+      xm_next = (t0 && tile + stride < ntiles && nline < L) ? ld_cg(in_nyq + nyq_index(sh, nline)) : make_float2(0.f, 0.f);
     }
     ok = __syncthreads_and(mbar_wait_bounded(&bar[s], parity, status));
     if (!ok) break;
@@ -247,14 +248,14 @@ __device__ __forceinline__ float2 load_pair(const void *rho, long o, int n2x, in
   if (BF16) {
     const uint16_t *r = (const uint16_t *)rho;
     if (even) {                                 // both values in one aligned 32-bit word
-      const uint32_t w = __ldg(reinterpret_cast<const unsigned int *>(r + o));
+      const uint32_t w = ld_cs(reinterpret_cast<const unsigned *>(r + o));
       return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
     }
-    return make_float2(bf16_to_f32(r[o]), n2x + 1 < nx ? bf16_to_f32(r[o + 1]) : 0.f);
+    return make_float2(bf16_to_f32(ld_cs(r + o)), n2x + 1 < nx ? bf16_to_f32(ld_cs(r + o + 1)) : 0.f);
   }
   const float *r = (const float *)rho;
-  if (even) return __ldcs(reinterpret_cast<const float2 *>(r + o));
-  return make_float2(r[o], n2x + 1 < nx ? r[o + 1] : 0.f);
+  if (even) return ld_cs(reinterpret_cast<const float2 *>(r + o));
+  return make_float2(ld_cs(r + o), n2x + 1 < nx ? ld_cs(r + o + 1) : 0.f);
 }
 
 // Four consecutive density values x[o .. o+3] (o a multiple of 4, row length a multiple
@@ -262,11 +263,11 @@ __device__ __forceinline__ float2 load_pair(const void *rho, long o, int n2x, in
 template <bool BF16>
 __device__ __forceinline__ float4 load_quad(const void *rho, long o) {
   if (BF16) {
-    const uint2 w = __ldg(reinterpret_cast<const uint2 *>((const uint16_t *)rho + o));
+    const uint2 w = ld_cs(reinterpret_cast<const uint2 *>((const uint16_t *)rho + o));
     return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u),
                        __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xffff0000u));
   }
-  return __ldcs(reinterpret_cast<const float4 *>((const float *)rho + o));
+  return ld_cs(reinterpret_cast<const float4 *>((const float *)rho + o));
 }
 
 // Groups with one family and one field (DIRECT) transform that family scaled by its
@@ -292,12 +293,13 @@ k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v
   constexpr int PADL = (M == 256) ? 1 : (CPT == 1 ? line_pad<T>() : 0);
   constexpr int LPB = THREADS / T, S = R1 * LD + PADL;
   static_assert(R1 * R2 == M && CPT >= 1 && CPT * T == R2 && CPT <= 2, "x forward config");
-  __shared__ float2 sm[LPB * S];
+  __shared__ __align__(16) float2 sm[LPB * S];
   // lines of up to 256 points: the M and 2M twiddles staged in shared memory (GaN layer
   // 0.233 -> 0.220 ms; for 512 points, eight lines per CTA, the staging costs more than
   // it saves: radial disk 0.036 -> 0.044 ms)
   constexpr bool STW = M <= 256;
-  __shared__ float2 stw[STW ? 3 * M : 1];
+  __shared__ __align__(16) float2 stw[STW ? 3 * M : 1];
+  pdl_trigger();
   const int t = threadIdx.x % T, lw = threadIdx.x / T;
   const long L = (long)sh.ny * sh.nz;
   const long N = L * sh.nx;
@@ -311,9 +313,10 @@ k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v
   const bool even = (sh.nx & 1) == 0;
   const bool quad = (sh.nx & 3) == 0;               // rows and column pairs 16-byte aligned
   if constexpr (STW) {
-    for (int i = threadIdx.x; i < M; i += THREADS) stw[i] = __ldg(tw + tw_offset(M) + i);
-    for (int i = threadIdx.x; i < 2 * M; i += THREADS) stw[M + i] = __ldg(tw + tw_offset(2 * M) + i);
+    stage_table<THREADS>(stw, tw + tw_offset(M), M, threadIdx.x);
+    stage_table<THREADS>(stw + M, tw + tw_offset(2 * M), 2 * M, threadIdx.x);
   }
+  pdl_wait();
   const float2 *twM = STW ? stw : tw + tw_offset(M);
   const float2 *tw2 = STW ? stw + M : tw + tw_offset(2 * M);
   const int ra = t, rb = t0 ? R1 / 2 : R1 - t;
@@ -379,7 +382,10 @@ k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v
     }
   }
   const float dscale = DIRECT ? col.coef[col.f0[g]][0] : 1.f;
-  if constexpr (STW) __syncthreads();                // twiddles staged
+  if constexpr (STW) {                               // twiddles staged
+    cp_async_wait_all();
+    __syncthreads();
+  }
 
 #pragma unroll
   for (int d = 0; d < NDM; ++d) {

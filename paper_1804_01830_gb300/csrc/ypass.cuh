@@ -52,6 +52,11 @@ __global__ void __launch_bounds__(NT) k_ypass_st(Shape sh, int nf, const float2 
   constexpr int R1 = YCfg<PY>::R1, R2 = YCfg<PY>::R2, ST = y_stride<PY, W>();
   extern __shared__ __align__(16) float2 sm[];              // y_smem_all<PY, W, INV, FULL>() values
   const int tid = threadIdx.x;
+  pdl_trigger();
+  constexpr bool STW = y_stw<PY, INV, FULL>();
+  float2 *stw = sm + y_smem<PY, W>();
+  if constexpr (STW) stage_table<NT>(stw, tw + tw_offset(PY), PY, tid);
+  pdl_wait();
   const int M = sh.M, nz = sh.nz;
   const int rows_in = INV ? PY : sh.ny;
   const int rows_out = INV ? sh.ny : PY;
@@ -94,10 +99,6 @@ __global__ void __launch_bounds__(NT) k_ypass_st(Shape sh, int nf, const float2 
       else sm[n * W + w] = make_float2(0.f, 0.f);
     }
   }
-  constexpr bool STW = y_stw<PY, INV, FULL>();
-  float2 *stw = sm + y_smem<PY, W>();
-  if constexpr (STW)
-    for (int i = tid; i < PY; i += NT) stw[i] = __ldg(tw + tw_offset(PY) + i);
   cp_async_wait_all();
   __syncthreads();
 

@@ -130,9 +130,10 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
   if (!nyq) zf_tile_of(tau, py, ktiles, &ky, &kxt);
   else nyq_idx = tau - tiles_main;
   const bool sw = sh.zs.xall && !nyq && ky > py / 2;   // works at the negated frequencies
+  pdl_trigger();
   float2 *twP = zsm + zf_smem0<PZ>(FE);
-  for (int i = tid; i < PZ; i += NT) twP[i] = __ldg(tw + tw_offset(PZ) + i);
-  __syncthreads();
+  stage_table<NT>(twP, tw + tw_offset(PZ), PZ, tid);
+  pdl_wait();
   // the stored tile this tile reads: its own, or py - ky for a negated-frequency tile
   const long st = nyq ? (long)(sh.zs.xall ? py / 2 + 1 : py) * ktiles + nyq_idx
                       : (long)(sw ? py - ky : ky) * ktiles + kxt;
@@ -161,8 +162,13 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
     const float2 *p = src + e * se + n2 * sz + w * sw1;
 #pragma unroll
     for (int n1 = 0; n1 < H; ++n1) {
-      ev[n1] = make_float2(0.f, 0.f);
-      if (n2 + R2 * n1 < nz) ev[n1] = __ldg(p + n1 * (R2 * sz));
+      const bool in = n2 + R2 * n1 < nz;
+      if constexpr (R1 == 32 && sizeof(GT) == 4) {   // (predicated, this instance spills: 0.91 -> 1.00 ms)
+        ev[n1] = make_float2(0.f, 0.f);
+        if (in) ev[n1] = ld_cg(p + n1 * (R2 * sz));
+      } else {                                // GaN batch, FP16 spectra: 0.85 -> 0.82 ms
+        ev[n1] = ld_cg_if(p + n1 * (R2 * sz), in);
+      }
     }
   };
   auto s1_finish = [&](int item, float2 (&ev)[H]) {
@@ -190,13 +196,22 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
   // The rows go first: requested ahead of them, the spectra delay them (GaN layer, with the
   // single pointer: 1.04 -> 0.93 ms).
   constexpr int IPR = ZF<PZ>::IPR;
+  auto table_ready = [&]() {                  // the twiddles have landed, for every thread
+    cp_async_wait_all();
+    __syncthreads();
+  };
+  constexpr bool ALL = NI >= NT;              // every thread has an item: wait behind its first rows
+  if constexpr (!ALL) table_ready();
   if constexpr (IPR == 2) {
     for (int item = tid; item < NI; item += 2 * NT) {
       float2 a[H], b[H];
       const bool two = item + NT < NI;
       s1_load(item, a);
       if (two) s1_load(item + NT, b);
-      if (item == tid) prefetch_spectra();
+      if (item == tid) {
+        prefetch_spectra();
+        if constexpr (ALL) table_ready();
+      }
       s1_finish(item, a);
       if (two) s1_finish(item + NT, b);
     }
@@ -209,7 +224,10 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
         ok[q] = q == 0 || item + q * NT < NI;
         if (ok[q]) s1_load(item + q * NT, a[q]);
       }
-      if (item == tid) prefetch_spectra();
+      if (item == tid) {
+        prefetch_spectra();
+        if constexpr (ALL) table_ready();
+      }
 #pragma unroll
       for (int q = 0; q < IPR; ++q)
         if (ok[q]) s1_finish(item + q * NT, a[q]);
@@ -301,10 +319,7 @@ cudaError_t launch_zfour(const Shape &sh, const float2 *im, const float2 *in, co
   constexpr int W = ZF<PZ>::W;
   if (sh.wz != W) return cudaErrorInvalidValue;
   const long tiles = ((long)sh.py * (sh.M / W) + sh.py / W) * sh.nb;
-  cudaError_t err = prep(k_zfour<PZ, FE, GT>, smem);
-  if (err != cudaSuccess) return err;
-  k_zfour<PZ, FE, GT><<<(unsigned)tiles, ZF<PZ>::NT, smem, s>>>(sh, im, in, ks, ksc, om, on, tw);
-  return cudaGetLastError();
+  return launch_pass<k_zfour<PZ, FE, GT>>(sh.early, (unsigned)tiles, ZF<PZ>::NT, smem, s, sh, im, in, ks, ksc, om, on, tw);
 }
 
 // FMIN, FMAX: the fewest and most fields the plan gives this padded z size.
