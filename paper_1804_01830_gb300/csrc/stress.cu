@@ -164,13 +164,13 @@ __global__ void k_stats_finish(const double *sums, long n, double inv_plane, flo
 
 // ------------------------------------------------------------ dispatch ------
 
-template <int M, bool BF16, bool DIRECT>
+template <int M, bool BF16, bool DIRECT, bool WIDE = false>
 cudaError_t launch_x_fwd_kind(const Shape &sh, const Collapse &col, const GroupList &gl, const void *rho,
                               float2 *om, float2 *on, const float2 *tw, cudaStream_t s) {
-  constexpr int LPB = xr::THREADS / (xr::FwdCfg<M>::R1 / 2);
+  constexpr int LPB = xr::THREADS / (xr::FwdCfg<M, WIDE>::R1 / 2);
   const long L = (long)sh.ny * sh.nz;
   dim3 grid((unsigned)((L + LPB - 1) / LPB), gl.n, sh.nb);
-  return launch_pass<xr::k_x_fwd_reg<M, BF16, DIRECT>>(sh.early, grid, xr::THREADS, 0, s, sh, col, gl, rho, om, on, tw);
+  return launch_pass<xr::k_x_fwd_reg<M, BF16, DIRECT, WIDE>>(sh.early, grid, xr::THREADS, 0, s, sh, col, gl, rho, om, on, tw);
 }
 
 // Groups with one family and one field transform that family directly; the others
@@ -191,6 +191,8 @@ cudaError_t launch_x_fwd(const Shape &sh, const Collapse &col, const void *rho, 
                : launch_x_fwd_kind<M, false, true>(sh, col, direct, rho, om, on, tw, s);
   }
   if (err == cudaSuccess && accum.n > 0) {
+    if constexpr (M == 128)
+      if (bf16 && sh.nx % 4 == 0) return launch_x_fwd_kind<M, true, false, true>(sh, col, accum, rho, om, on, tw, s);
     err = bf16 ? launch_x_fwd_kind<M, true, false>(sh, col, accum, rho, om, on, tw, s)
                : launch_x_fwd_kind<M, false, false>(sh, col, accum, rho, om, on, tw, s);
   }

@@ -34,13 +34,17 @@ template <> struct InvCfg<512> { static constexpr int R1 = 16, R2 = 32; };
 // Forward: R1 points per column of which the first R1 / 2 are non-zero (the padded
 // half of the line), R2 columns, T = R1 / 2 threads per line, each owning rows t and
 // R1 - t of the second stage (thread 0: rows 0 and R1 / 2).
-template <int M> struct FwdCfg;
-template <> struct FwdCfg<16>  { static constexpr int R1 = 4,  R2 = 4; };
-template <> struct FwdCfg<32>  { static constexpr int R1 = 8,  R2 = 4; };
-template <> struct FwdCfg<64>  { static constexpr int R1 = 8,  R2 = 8; };
-template <> struct FwdCfg<128> { static constexpr int R1 = 16, R2 = 8; };
-template <> struct FwdCfg<256> { static constexpr int R1 = 16, R2 = 16; };
-template <> struct FwdCfg<512> { static constexpr int R1 = 32, R2 = 16; };
+// WIDE: eight-value runs per thread (four columns) instead of two-value ones, for BF16 rows
+// that are summed over families: 128x128x128, four sets, 18 families, 0.346 -> 0.193 ms; with
+// FP32 rows, or rows not a multiple of 4 values, it is slower (0.059 -> 0.074 ms a set).
+template <int M, bool WIDE = false> struct FwdCfg;
+template <> struct FwdCfg<16, false>  { static constexpr int R1 = 4,  R2 = 4; };
+template <> struct FwdCfg<32, false>  { static constexpr int R1 = 8,  R2 = 4; };
+template <> struct FwdCfg<64, false>  { static constexpr int R1 = 8,  R2 = 8; };
+template <> struct FwdCfg<128, false> { static constexpr int R1 = 16, R2 = 8; };
+template <> struct FwdCfg<128, true> { static constexpr int R1 = 8, R2 = 16; };
+template <> struct FwdCfg<256, false> { static constexpr int R1 = 16, R2 = 16; };
+template <> struct FwdCfg<512, false> { static constexpr int R1 = 32, R2 = 16; };
 
 constexpr int THREADS = 128;
 
@@ -278,21 +282,21 @@ __device__ __forceinline__ float4 load_quad(const void *rho, long o) {
 // SM), and bound to three it takes 163 and runs 18% slower.  512 points: direct groups
 // four (radial disk 0.042 ms left free at 207 registers, 0.036 at three or four); summed
 // families the compiler's choice (254 registers; bound to three they spill 312 bytes).
-template <int M, bool DIRECT> constexpr int x_fwd_ctas() {
-  return M == 256 ? 3 : (M == 128 ? 4 : (M == 512 && DIRECT ? 4 : 1));
+template <int M, bool DIRECT, bool WIDE> constexpr int x_fwd_ctas() {
+  return M == 256 ? 3 : (M == 128 ? (WIDE ? 3 : 4) : (M == 512 && DIRECT ? 4 : 1));
 }
 
-template <int M, bool BF16, bool DIRECT>
-__global__ void __launch_bounds__(THREADS, (x_fwd_ctas<M, DIRECT>()))
+template <int M, bool BF16, bool DIRECT, bool WIDE>
+__global__ void __launch_bounds__(THREADS, (x_fwd_ctas<M, DIRECT, WIDE>()))
 k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v, float2 *__restrict__ out_main,
             float2 *__restrict__ out_nyq, const float2 *__restrict__ tw) {
-  constexpr int R1 = FwdCfg<M>::R1, R2 = FwdCfg<M>::R2, T = R1 / 2, CPT = R2 / T, H = R1 / 2;
+  constexpr int R1 = FwdCfg<M, WIDE>::R1, R2 = FwdCfg<M, WIDE>::R2, T = R1 / 2, CPT = R2 / T, H = R1 / 2;
   // thread t owns the adjacent columns n2 = CPT t + q; row stride and line shift keep
   // the shared-memory stages free of bank conflicts (2-way left for M = 16, 64)
   constexpr int LD = (M == 256) ? R2 + 2 : R2 + 1;
-  constexpr int PADL = (M == 256) ? 1 : (CPT == 1 ? line_pad<T>() : 0);
+  constexpr int PADL = (M == 256 || WIDE) ? 1 : (CPT == 1 ? line_pad<T>() : 0);
   constexpr int LPB = THREADS / T, S = R1 * LD + PADL;
-  static_assert(R1 * R2 == M && CPT >= 1 && CPT * T == R2 && CPT <= 2, "x forward config");
+  static_assert(R1 * R2 == M && CPT >= 1 && CPT * T == R2 && CPT <= 4, "x forward config");
   __shared__ __align__(16) float2 sm[LPB * S];
   // lines of up to 256 points: the M and 2M twiddles staged in shared memory (GaN layer
   // 0.233 -> 0.220 ms; for 512 points, eight lines per CTA, the staging costs more than
@@ -340,18 +344,20 @@ k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v
       const int fi = col.f0[g] + f;
       const long base = set_off + (long)col.fam[fi] * N + line * sh.nx;
       float2 v[CPT][H];
-      if (CPT == 2 && quad) {                 // both columns' pairs in one 16-byte (8 for bf16) load
+      if (CPT >= 2 && quad) {                 // two columns' pairs in one 16-byte (8 for bf16) load
 #pragma unroll
-        for (int n1 = 0; n1 < H; ++n1) {
-          const int n = CPT * t + R2 * n1;    // even; nxh even, so n + 1 < nxh with n
-          if (n < nxh) {
-            const float4 x = load_quad<BF16>(rho_v, base + 2 * n);
-            v[0][n1] = make_float2(x.x, x.y);
-            v[CPT - 1][n1] = make_float2(x.z, x.w);
-          } else {
-            v[0][n1] = v[CPT - 1][n1] = make_float2(0.f, 0.f);
+        for (int q = 0; q + 1 < CPT; q += 2)
+#pragma unroll
+          for (int n1 = 0; n1 < H; ++n1) {
+            const int n = CPT * t + q + R2 * n1;       // even; nxh even, so n + 1 < nxh with n
+            if (n < nxh) {
+              const float4 x = load_quad<BF16>(rho_v, base + 2 * n);
+              v[q][n1] = make_float2(x.x, x.y);
+              v[q + 1][n1] = make_float2(x.z, x.w);
+            } else {
+              v[q][n1] = v[q + 1][n1] = make_float2(0.f, 0.f);
+            }
           }
-        }
       } else {
 #pragma unroll
         for (int q = 0; q < CPT; ++q)
