@@ -113,6 +113,9 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
             float2 *out_main, float2 *out_nyq, const float2 *tw) {
   constexpr int R1 = ZF<PZ>::R1, R2 = ZF<PZ>::R2, W = ZF<PZ>::W, NT = ZF<PZ>::NT;
   constexpr int SK = ZF<PZ>::SK, SY = ZF<PZ>::SY, H = R1 / 2;
+  // packed butterflies in stages 1 and 3; stage 2 keeps rho^ in every register it has, and
+  // pairs would spill (GaN layer 0.954 against 0.917 ms)
+  constexpr bool PK1 = true, PK2 = false, PK3 = true;
   extern __shared__ __align__(16) float2 zsm[];
   const int tid = threadIdx.x;
   const int M = sh.M, py = sh.py, nz = sh.nz;
@@ -181,8 +184,8 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
     float2 od[H];
 #pragma unroll
     for (int n1 = 0; n1 < H; ++n1) od[n1] = rot_const<false>(ev[n1], n1, R1);
-    dft_reg<H, false>(ev);                    // outputs k1 = 2 j
-    dft_reg<H, false>(od);                    // outputs k1 = 2 j + 1
+    dft_reg<H, false, PK1>(ev);                    // outputs k1 = 2 j
+    dft_reg<H, false, PK1>(od);                    // outputs k1 = 2 j + 1
     float2 *T = zsm + (long)e * R1 * SK + n2 * W + w;
 #pragma unroll
     for (int j = 0; j < H; ++j) {
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
   for (int e = 0; e < FE; ++e) {
 #pragma unroll
     for (int n2 = 0; n2 < R2; ++n2) f[e][n2] = zsm[((long)e * R1 + k1) * SK + n2 * W + w];
-    dft_reg<R2, false>(f[e]);
+    dft_reg<R2, false, PK2>(f[e]);
   }
   __syncthreads();                            // T is read: Y takes its space
 #pragma unroll 1
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
 #pragma unroll
       for (int k2 = 0; k2 < R2; ++k2) s[k2] = cmadd_i(s[k2], lt.get(e - PF, k2, sc), f[e][k2]);
     }
-    dft_reg<R2, true>(s);                     // index a of n = a + R2 b
+    dft_reg<R2, true, PK2>(s);                     // index a of n = a + R2 b
     float2 *Y = zsm + (long)c * R2 * SY + k1 * W + w;
     Y[0] = s[0];
 #pragma unroll
@@ -292,8 +295,8 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
       ev[j] = Y[(2 * j) * W];
       od[j] = Y[(2 * j + 1) * W];
     }
-    dft_reg<H, true>(ev);
-    dft_reg<H, true>(od);
+    dft_reg<H, true, PK3>(ev);
+    dft_reg<H, true, PK3>(od);
     float2 *dst = nyq ? out_nyq + ((long)c * py + nyq_idx * W + wc) * nz
                       : out_main + ((long)c * nz * py + ky) * M + kxt * W + wc;
 #pragma unroll
