@@ -247,6 +247,7 @@ int make_plan(dds_ctx *ctx) {
   sh.wz = 0;
   sh.zreg_g = 0;
   sh.zfour = 0;
+  sh.ztile = 0;
   sh.nb = 1;
   sh.early = 0;
   sh.yxf = ctx->yx_fused ? yx_inv_cluster(sh) : 0;
@@ -281,6 +282,7 @@ int make_plan(dds_ctx *ctx) {
                   "(pz %d, %d fields)", sh.pz, sh.fe);
     sh.zfour = 1;
     sh.wz = fw;
+    sh.ztile = sh.py <= 512 ? 1 : 0;
     zfour_symmetry(ctx->field_t.data(), ctx->field_b.data(), sh.fe, &sh);
     ctx->shape = sh;
     return DDS_OK;

@@ -49,6 +49,13 @@ struct Shape {
   int wz;             // columns per tile of the fused z pass (shared-memory variant)
   int zreg_g;         // > 0: register-only z pass, pz = 16 * zreg_g, zreg_g lanes per column
   int zfour;          // 1: three-stage register z pass (wz = zfour_width(pz))
+  // zfour: after the forward y pass the main array is [ky][z tile][field][z][column of the
+  // tile] instead of [field][z][ky][kx], so that a z tile reads one contiguous block: its
+  // 64-byte row pieces otherwise lie a plane apart, one to a DRAM page (GaN layer, z pass 0.92
+  // -> 0.82 ms for 0.03 ms more in the y pass; 90x77x200 0.41 -> 0.36 ms).  Not for 1024 rows,
+  // whose y tiles are four columns wide: 32-byte writes cost the y pass more (512x512x64, two
+  // sets, 0.90 -> 1.35 ms) than the z pass gains.
+  int ztile;
   int nb;             // density sets evaluated together (batch); fields are [b][e], outputs [b][c]
   ZSym zs;            // zfour: stored-spectrum symmetries and layout
   int early;          // launches may start before the kernel ahead of them has finished

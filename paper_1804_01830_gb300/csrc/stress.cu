@@ -16,7 +16,7 @@
 // The Nyquist column kx = M of the half spectrum travels in separate small
 // arrays.  Layouts (complex):
 //   after x_fwd : main [e][z][y][kx < M],  nyq [e][y][z]
-//   after y_fwd : main [e][z][ky][kx],     nyq [e][ky][z]
+//   after y_fwd : main [e][z][ky][kx] (or by z tile, Shape::ztile), nyq [e][ky][z]
 //   after z     : main [c][z][ky][kx],     nyq [c][ky][z]
 //   after y_inv : main [c][z][y][kx],      nyq [c][y][z]
 // The y passes keep W columns interleaved in shared memory (lanes across

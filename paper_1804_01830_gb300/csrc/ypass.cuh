@@ -65,24 +65,33 @@ __global__ void __launch_bounds__(NT) k_ypass_st(Shape sh, int nf, const float2 
   const long tau = blockIdx.x;
   const float2 *in;
   float2 *out;
-  long rs;
+  long rs, ro;                                // row strides of the input and the output
   int ncols;
+  const int wo = tid % W;                     // the column this thread stores
+  static_assert(NT % W == 0, "a thread stores one column");
   const bool main_tile = tau < tiles_main;
   if (main_tile) {
     const int e = (int)(tau / (nz * ktiles));
     const long r = tau - (long)e * nz * ktiles;
     const int z = (int)(r / ktiles), kt = (int)(r - (long)z * ktiles);
     in = in_main + ((long)(e * nz + z) * rows_in) * M + kt * W;
-    out = out_main + ((long)(e * nz + z) * rows_out) * M + kt * W;
     rs = M;
+    if (!INV && sh.ztile) {                   // [set][ky][z tile][field][z][column of the tile]
+      const int b = e / sh.fe, kx = kt * W + wo, wz = sh.wz, rows = sh.fe * nz;
+      out = out_main + ((long)b * rows_out * (M / wz) + kx / wz) * rows * wz + ((e - b * sh.fe) * nz + z) * wz + kx % wz;
+      ro = (long)rows * M;
+    } else {
+      out = out_main + ((long)(e * nz + z) * rows_out) * M + kt * W + wo;
+      ro = M;
+    }
     ncols = W;
   } else {
     const long t2 = tau - tiles_main;
     const int ztiles = (nz + W - 1) / W;
     const int e = (int)(t2 / ztiles), zt = (int)(t2 - (long)e * ztiles);
     in = in_nyq + (long)e * rows_in * nz + zt * W;
-    out = out_nyq + (long)e * rows_out * nz + zt * W;
-    rs = nz;
+    out = out_nyq + (long)e * rows_out * nz + zt * W + wo;
+    rs = ro = nz;
     ncols = min(W, nz - zt * W);
   }
   // stage the rows: element (n, w) at sm[n W + w]
@@ -169,7 +178,7 @@ __global__ void __launch_bounds__(NT) k_ypass_st(Shape sh, int nf, const float2 
 #pragma unroll
       for (int k2 = 0; k2 < K2; ++k2) {
         const int k = k1 + R1 * k2;
-        if (k < rows_out) __stcs(out + (long)k * rs + w, y[k2]);
+        if (k < rows_out) __stcs(out + k * ro, y[k2]);
       }
     }
   }

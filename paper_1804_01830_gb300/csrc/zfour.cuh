@@ -158,8 +158,12 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
   // kinds of tile: a choice between two loads per element compiles to branches, which
   // keep the loads of an item from being in flight together (padded z 128, 512x512x64
   // with two sets: 5.14 -> 3.21 ms)
-  const float2 *src = nyq ? in_nyq + (long)nyq_idx * W * nz : in_main + (long)ky * M + kxt * W;
-  const long sz = nyq ? 1 : (long)py * M, sw1 = nyq ? nz : 1, se = (long)nz * py * (nyq ? 1 : M);
+  const bool own = sh.ztile;                  // the tile's rows lie together
+  const float2 *src = nyq   ? in_nyq + (long)nyq_idx * W * nz
+                      : own ? in_main + ((long)ky * ktiles + kxt) * (FE * nz * W)
+                            : in_main + (long)ky * M + kxt * W;
+  const long sz = nyq ? 1 : own ? (long)W : (long)py * M, sw1 = nyq ? nz : 1;
+  const long se = (long)nz * (nyq ? (long)py : own ? (long)W : (long)py * M);
   auto s1_load = [&](int item, float2 (&ev)[H]) {
     const int e = item / (R2 * W), r = item - e * (R2 * W), n2 = r / W, w = r - n2 * W;
     const float2 *p = src + e * se + n2 * sz + w * sw1;
@@ -297,6 +301,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
     }
     dft_reg<H, true, PK3>(ev);
     dft_reg<H, true, PK3>(od);
+    const long so = nyq ? 1 : (long)py * M;
     float2 *dst = nyq ? out_nyq + ((long)c * py + nyq_idx * W + wc) * nz
                       : out_main + ((long)c * nz * py + ky) * M + kxt * W + wc;
 #pragma unroll
@@ -309,7 +314,7 @@ __global__ void __launch_bounds__(ZF<PZ>::NT, PZ == 512 ? 2 : 512 / ZF<PZ>::NT)
         // and they leave L2 to the mirror tiles' spectra (1.049 -> 1.041 ms); streaming
         // loads of the density rows cost more (1.088 ms), since neighbouring tiles share
         // their 128-byte lines
-        __stcs(dst + z * sz, v);
+        __stcs(dst + z * so, v);
       }
     }
   }
