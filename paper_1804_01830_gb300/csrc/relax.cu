@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include "dds_internal.h"
+#include "stress_common.cuh"
 
 namespace dds {
 namespace {
@@ -85,7 +86,7 @@ __global__ void k_relax_prep(RelaxCoef r, const float *__restrict__ sig, float *
 }
 
 // The march over the film, shared by the step and the stress kernels.  256 threads take a
-// tile of 64 x 8 columns, two x-adjacent cells per thread, up a chunk of layers.  Planes of
+// tile of 64 x 8 (or 32 x 16) columns, two x-adjacent cells per thread, up a chunk of layers.  Planes of
 // u (three components, one-cell halo) arrive in a ring of shared-memory slots by
 // cp.async, up to three layers ahead of the layer that uses them; ghost planes are evaluated
 // into their slot.  A plane is read from shared memory once, when it is the one above the
@@ -101,11 +102,18 @@ __global__ void k_relax_prep(RelaxCoef r, const float *__restrict__ sig, float *
 // rate; deeper rings and one cell per thread measured the same or slower.  Step, GaN grid
 // 256x256x128: 94 -> 77 us, 512x512x16: 61 -> 49 us; total stress: 442 -> 105 us and 226 ->
 // 63 us (it evaluated ghost layers and offsets per value before).
-constexpr int TX = 64, TY = 8, PX = TX / 2, HY = TY + 2, NTM = PX * TY, RING = 4;
-constexpr int X0 = 4, LD = TX + 8;                 // column x of the tile at X0 + x: 16-byte aligned rows
-constexpr int CS = HY * LD, PLANE = 3 * CS;
-// a slot: one plane, and the threads' own inputs (NC fields) of the layer below it
-template <int NC> __host__ __device__ constexpr int slot_floats() { return PLANE + NC * 2 * NTM; }
+constexpr int NTM = 256, RING = 4, X0 = 4;         // column x of the tile at X0 + x: 16-byte aligned rows
+template <int PX> struct March {                   // PX threads along x
+  static constexpr int TX = 2 * PX, TY = NTM / PX, HY = TY + 2, LD = TX + 8, CS = HY * LD, PLANE = 3 * CS;
+  // a slot: one plane, and the threads' own inputs (NC fields) of the layer below it
+  template <int NC> static constexpr int slot_floats() { return PLANE + NC * 2 * NTM; }
+};
+
+__device__ __forceinline__ float ld_cg1(const float *p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
 
 __device__ __forceinline__ int mod(int i, int n) { return ((i % n) + n) % n; }
 
@@ -133,7 +141,9 @@ struct Stage {
   int src[3], dst[3];
   int col;                 // first column of the groups
 };
+template <int PX>
 __device__ __forceinline__ Stage make_stage(const RelaxCoef &r, int i0, int j0) {
+  constexpr int TX = March<PX>::TX, HY = March<PX>::HY, LD = March<PX>::LD;
   constexpr int G = TX / 4, ROWS = 3 * HY, PASS = NTM / G;
   static_assert(ROWS <= 2 * PASS && 2 * ROWS <= NTM, "two passes over the rows, one over the halo columns");
   auto film = [&](int row, int i) { return (int)cidx(r, row / HY, 0, mod(j0 + row % HY - 1, r.ny), i); };
@@ -158,8 +168,10 @@ __device__ __forceinline__ Stage make_stage(const RelaxCoef &r, int i0, int j0) 
 //   u_z: (phi_zz - nu (du_x/dx + du_y/dy)) / (1 - nu).  A thread evaluates
 // all components at its three positions with every load in flight: one position and
 // component at a time, the surface chunks waited 8 times a memory latency for it.
-__device__ __forceinline__ void ghost_plane(const RelaxCoef &r, const float *__restrict__ u,
-                                            const float *__restrict__ phi, int i0, int j0, int k, float *pl) {
+template <int PX>
+__device__ __forceinline__ void ghost_plane(const RelaxCoef &r, const float *u, const float *phi, int i0, int j0, int k,
+                                            float *pl) {
+  constexpr int TX = March<PX>::TX, HY = March<PX>::HY, LD = March<PX>::LD, CS = March<PX>::CS;
   constexpr int W = TX + 2, NP = (HY * W + NTM - 1) / NTM;
   const bool top = k >= r.nz;
   const int plane = r.ny * r.nx, cs = r.nz * plane;
@@ -176,17 +188,17 @@ __device__ __forceinline__ void ghost_plane(const RelaxCoef &r, const float *__r
     const int on = wrap(j + 1, r.ny) * r.nx + i, os = wrap(j - 1, r.ny) * r.nx + i;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      in[e][c] = __ldg(un + c * cs + o);
-      f[e][c] = __ldg(ph + c * plane + o);
+      in[e][c] = ld_cg1(un + c * cs + o);
+      f[e][c] = ld_cg1(ph + c * plane + o);
     }
-    zx[e][0] = __ldg(us + 2 * cs + oe);
-    zx[e][1] = __ldg(us + 2 * cs + ow);
-    zy[e][0] = __ldg(us + 2 * cs + on);
-    zy[e][1] = __ldg(us + 2 * cs + os);
-    xx[e][0] = __ldg(us + oe);
-    xx[e][1] = __ldg(us + ow);
-    yy[e][0] = __ldg(us + cs + on);
-    yy[e][1] = __ldg(us + cs + os);
+    zx[e][0] = ld_cg1(us + 2 * cs + oe);
+    zx[e][1] = ld_cg1(us + 2 * cs + ow);
+    zy[e][0] = ld_cg1(us + 2 * cs + on);
+    zy[e][1] = ld_cg1(us + 2 * cs + os);
+    xx[e][0] = ld_cg1(us + oe);
+    xx[e][1] = ld_cg1(us + ow);
+    yy[e][0] = ld_cg1(us + cs + on);
+    yy[e][1] = ld_cg1(us + cs + os);
   }
 #pragma unroll
   for (int e = 0; e < NP; ++e) {
@@ -201,10 +213,9 @@ __device__ __forceinline__ void ghost_plane(const RelaxCoef &r, const float *__r
 
 // Starts plane k (a layer, or a ghost layer at -1 and nz) into slot pl, in the current copy group.
 // vec: rows of u are 16-byte aligned (whole groups of four).
-template <bool FULL>
-__device__ __forceinline__ void start_plane(const RelaxCoef &r, const float *__restrict__ u,
-                                            const float *__restrict__ phi, const Stage &st, int i0, int j0, int k,
-                                            bool vec, float *pl) {
+template <int PX, bool FULL>
+__device__ __forceinline__ void start_plane(const RelaxCoef &r, const float *u, const float *phi, const Stage &st, int i0,
+                                            int j0, int k, bool vec, float *pl) {
   if (k >= 0 && k < r.nz) {
     const float *layer = u + (long)k * (r.ny * r.nx);
     if constexpr (FULL) {
@@ -230,7 +241,7 @@ __device__ __forceinline__ void start_plane(const RelaxCoef &r, const float *__r
     }
     if (st.src[2] >= 0) cp_async4(pl + st.dst[2], layer + st.src[2]);
   } else {
-    ghost_plane(r, u, phi, i0, j0, k, pl);
+    ghost_plane<PX>(r, u, phi, i0, j0, k, pl);
   }
 }
 
@@ -257,8 +268,9 @@ __device__ __forceinline__ Row load_row(const float *p) {
   return v;
 }
 
-template <bool STEP>
+template <int PX, bool STEP>
 __device__ __forceinline__ void read_plane(const RelaxCoef &r, const float *p, PlaneTerms &t) {
+  constexpr int CS = March<PX>::CS, LD = March<PX>::LD;
   float2 xs[3], ys[3], cross[2];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -291,25 +303,27 @@ __device__ __forceinline__ void read_plane(const RelaxCoef &r, const float *p, P
 
 // STEP: one explicit step, out[3] = u + dt (navier(u) + f), gin[3] = dt f.  Otherwise the
 // total stress, out[6] = gin[6] + lambda div u delta + mu (du_a/db + du_b/da).
-template <bool STEP, bool FULL>
+template <int PX, bool STEP, bool FULL>
 __global__ void __launch_bounds__(NTM, 2)
-k_relax_march(RelaxCoef r, const float *__restrict__ u, const float *gin, const float *__restrict__ phi, float *out,
-              int kz, int vec) {
-  constexpr int NC = STEP ? 3 : 6;
-  constexpr int SLOT = slot_floats<NC>();
+k_relax_march(RelaxCoef r, const float *u, const float *gin, const float *phi, float *out, int kz, int vec) {
+  using C = March<PX>;
+  constexpr int TX = C::TX, TY = C::TY, LD = C::LD, PLANE = C::PLANE, NC = STEP ? 3 : 6;
+  constexpr int SLOT = C::template slot_floats<NC>();
   extern __shared__ __align__(16) float ring[];
   const int tx = threadIdx.x % PX, ty = threadIdx.x / PX;
   const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY, i = i0 + 2 * tx;
   const int kb = blockIdx.z * kz, ke = min(kb + kz, r.nz);
   const bool live = FULL || (i < r.nx && j0 + ty < r.ny), second = FULL || i + 1 < r.nx;
   const int plane = r.ny * r.nx, cstride = r.nz * plane, own = (j0 + ty) * r.nx + i;
-  const Stage st = make_stage(r, i0, j0);
+  pdl_trigger();
+  const Stage st = make_stage<PX>(r, i0, j0);
+  pdl_wait();                                      // u of the step before
   const int mine = (ty + 1) * LD + X0 + 2 * tx, own_in = PLANE + 2 * threadIdx.x;
   // one copy group, into slot q: plane k and the cells' inputs of layer k - 1 (nothing past
   // the plane above the chunk)
   auto start = [&](int k, int q) {
     if (k <= ke) {
-      start_plane<FULL>(r, u, phi, st, i0, j0, k, vec, ring + q * SLOT);
+      start_plane<PX, FULL>(r, u, phi, st, i0, j0, k, vec, ring + q * SLOT);
       if (live && k > kb) {
         float *dst = ring + q * SLOT + own_in;
         const int o = own + (k - 1) * plane;
@@ -337,7 +351,7 @@ k_relax_march(RelaxCoef r, const float *__restrict__ u, const float *gin, const 
     start(k + RING, sq == 0 ? RING - 1 : sq - 1);
     const float *slot = ring + sq * SLOT;
     sq = sq == RING - 1 ? 0 : sq + 1;
-    read_plane<STEP>(r, slot + mine, t[D]);
+    read_plane<PX, STEP>(r, slot + mine, t[D]);
     float2 g[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) g[c] = *reinterpret_cast<const float2 *>(slot + own_in + 2 * NTM * c);
@@ -379,8 +393,8 @@ k_relax_march(RelaxCoef r, const float *__restrict__ u, const float *gin, const 
   for (int q = 0; q < RING; ++q) start(kb - 1 + q, q);
   asm volatile("cp.async.wait_group %0;\n" ::"n"(RING - 2) : "memory");
   __syncthreads();
-  read_plane<STEP>(r, ring + mine, t[0]);
-  read_plane<STEP>(r, ring + SLOT + mine, t[1]);
+  read_plane<PX, STEP>(r, ring + mine, t[0]);
+  read_plane<PX, STEP>(r, ring + SLOT + mine, t[1]);
   __syncthreads();                                 // slot 0 is read
   start(kb - 1 + RING, 0);
   using I0 = std::integral_constant<int, 0>;
@@ -426,30 +440,38 @@ RelaxCoef relax_coef(const dds_ctx *ctx, double *dt_out) {
   return r;
 }
 
-template <bool STEP>
-cudaError_t launch_march(const RelaxCoef &r, const float *u, const float *in, const float *phi, float *out,
-                         cudaStream_t s) {
+template <int PX, bool STEP>
+cudaError_t launch_march_px(const RelaxCoef &r, const float *u, const float *in, const float *phi, float *out, bool early,
+                            cudaStream_t s) {
+  using C = March<PX>;
   // Layers per chunk: 16, or 8 or 4 where that would leave CTA slots (two per SM) idle.
   // Longer chunks restart the march less often, but leave an emptier last wave (step on
   // 256x256x128: 8 / 16 / 32 / 64 layers 82 / 77 / 82 / 81 us; 512x512x16: 8 / 16 layers
-  // 49 / 51 us; 100x90x40: 4 / 8 / 16 layers
-  // 11.9 / 12.3 / 20 us).
+  // 49 / 51 us; 100x90x40: 4 / 8 / 16 layers 9 / 12 / 20 us).
   int dev = 0, sms = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
-  const long tiles = (long)((r.nx + TX - 1) / TX) * ((r.ny + TY - 1) / TY);
+  const long tiles = (long)((r.nx + C::TX - 1) / C::TX) * ((r.ny + C::TY - 1) / C::TY);
   const int kz = tiles * ((r.nz + 15) / 16) >= 4 * sms ? 16 : (tiles * ((r.nz + 7) / 8) >= 2 * sms ? 8 : 4);
-  const dim3 grid((unsigned)((r.nx + TX - 1) / TX), (unsigned)((r.ny + TY - 1) / TY), (unsigned)((r.nz + kz - 1) / kz));
+  const dim3 grid((unsigned)((r.nx + C::TX - 1) / C::TX), (unsigned)((r.ny + C::TY - 1) / C::TY),
+                  (unsigned)((r.nz + kz - 1) / kz));
   const int vec = r.nx % 4 == 0 && ((uintptr_t)u & 15) == 0;
-  const bool full = vec && r.nx % TX == 0 && r.ny % TY == 0 && (((uintptr_t)in | (uintptr_t)out) & 7) == 0;
-  const size_t smem = sizeof(float) * RING * slot_floats<STEP ? 3 : 6>();
-  auto kernel = full ? k_relax_march<STEP, true> : k_relax_march<STEP, false>;
-  err = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-  if (err == cudaSuccess) err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  kernel<<<grid, NTM, smem, s>>>(r, u, in, phi, out, kz, vec);
-  return cudaGetLastError();
+  const bool full = vec && r.nx % C::TX == 0 && r.ny % C::TY == 0 && (((uintptr_t)in | (uintptr_t)out) & 7) == 0;
+  const size_t smem = sizeof(float) * RING * C::template slot_floats<STEP ? 3 : 6>();
+  if (full) return launch_pass<k_relax_march<PX, STEP, true>>(early, grid, NTM, smem, s, r, u, in, phi, out, kz, vec);
+  return launch_pass<k_relax_march<PX, STEP, false>>(early, grid, NTM, smem, s, r, u, in, phi, out, kz, vec);
+}
+
+template <bool STEP>
+cudaError_t launch_march(const RelaxCoef &r, const float *u, const float *in, const float *phi, float *out, bool early,
+                         cudaStream_t s) {
+  // tiles of 64 x 8 columns, or of 32 x 16 where those overhang the rows less (step on
+  // 160x160x32 15.9 -> 11.9 us, 32x512x4 9.2 -> 6.1 us; on 256x256x128 they take 87 against
+  // 76 us)
+  const int w64 = (r.nx + 63) / 64 * 64, w32 = (r.nx + 31) / 32 * 32;
+  return w32 < w64 ? launch_march_px<16, STEP>(r, u, in, phi, out, early, s)
+                   : launch_march_px<32, STEP>(r, u, in, phi, out, early, s);
 }
 
 }  // namespace
@@ -468,11 +490,15 @@ int enqueue_relax(dds_ctx *ctx, const float *sig, float *u, int n_steps, float *
     }
     ctx->relax_n = need;
   }
+  // a captured chain keeps full dependencies (see the evaluation's passes)
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t err = cudaStreamIsCapturing(s, &capture);
+  const bool early = err == cudaSuccess && capture == cudaStreamCaptureStatusNone;
   float *gf = ctx->relax_buf, *tmp = gf + 3 * N, *phi = tmp + 3 * N;
   const dim3 blk(32, 4, 1);
   const dim3 grid((unsigned)((r.nx + 31) / 32), (unsigned)((r.ny + 3) / 4), (unsigned)r.nz);
   k_relax_prep<<<grid, blk, 0, s>>>(r, sig, gf, phi);
-  cudaError_t err = cudaGetLastError();
+  if (err == cudaSuccess) err = cudaGetLastError();
   // ping-pong so that the last step writes into u
   float *a = u, *b = tmp;
   if (n_steps % 2 == 1 && err == cudaSuccess) {
@@ -481,10 +507,10 @@ int enqueue_relax(dds_ctx *ctx, const float *sig, float *u, int n_steps, float *
     b = u;
   }
   for (int t = 0; t < n_steps && err == cudaSuccess; ++t) {
-    err = launch_march<true>(r, a, gf, phi, b, s);
+    err = launch_march<true>(r, a, gf, phi, b, early, s);
     std::swap(a, b);
   }
-  if (err == cudaSuccess && sig_tot) err = launch_march<false>(r, u, sig, phi, sig_tot, s);
+  if (err == cudaSuccess && sig_tot) err = launch_march<false>(r, u, sig, phi, sig_tot, early, s);
   if (err != cudaSuccess) return fail(ctx, DDS_ERR_CUDA, "relax: kernel launch failed: %s", cudaGetErrorString(err));
   return DDS_OK;
 }

@@ -1,4 +1,4 @@
-"""The relaxation's march at the edges of its tiles (64 x 8 columns), chunks (4, 8 and 16
+"""The relaxation's march at the edges of its tiles (64 x 8 and 32 x 16 columns), chunks (4, 8 and 16
 layers) and copies (16-byte, 8-byte and single values): every shape against the FP64
 oracle after a few steps, with the bounds of the step-for-step test (1e-6 + K 2^-24
 relative L2 after K steps; the total stress relative to its largest component)."""
@@ -17,7 +17,8 @@ TOL = 1e-6 + STEPS * 2.0 ** -24
 
 
 @pytest.mark.parametrize("shape", [(2, 8, 64), (4, 9, 65), (5, 7, 63), (16, 16, 128), (17, 1, 1), (18, 3, 2), (33, 8, 68),
-                                   (9, 8, 60), (65, 72, 192), (40, 90, 100), (17, 200, 512)])
+                                   (9, 8, 60), (65, 72, 192), (40, 90, 100), (17, 200, 512),
+                                   (6, 16, 32), (9, 17, 31), (4, 33, 96), (21, 15, 160)])
 @pytest.mark.parametrize("shift", [0, 1])            # first value of u, load and total off 16-byte alignment
 def test_tile_edges(shape, shift):
     import paper_1804_01830_gb300 as dds
