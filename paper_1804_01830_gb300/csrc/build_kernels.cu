@@ -48,8 +48,10 @@ struct Box {
   double hl, f;
 };
 
-// NF fields of one line direction: what their coefficients share.
-template <int NF> struct Fields {
+// NF fields of one line direction: what their coefficients share.  TZ: t = (0, 0, 1) exactly
+// (the vertical dislocations of the paper's layers); the terms that vanish are then left
+// out: 64x64x8 with 15 replica shells, two fields, table 15.4 -> 11 ms.
+template <int NF, bool TZ> struct Fields {
   V3 t;
   V3 b[NF], w[NF];          // Burgers vectors, b x t
   double k1;                // 1 / (1 - nu)
@@ -73,12 +75,12 @@ template <int NF> struct Fields {
 // of evaluating Eq. 6 per end and field (GaN layer, five fields: tables 234 -> 12.4 ms
 // with the offsets the symmetries leave; 15 replica shells on 64x64x8, two fields: 374 ->
 // 15.4 ms).  The observer at the centre gives 0.
-template <int NF>
-__device__ __forceinline__ void box_add(const Fields<NF> &F, V3 r, const Box &box, double weight, double (&acc)[NF][6]) {
+template <int NF, bool TZ>
+__device__ __forceinline__ void box_add(const Fields<NF, TZ> &F, V3 r, const Box &box, double weight, double (&acc)[NF][6]) {
   if (r.x == 0.0 && r.y == 0.0 && r.z == 0.0) return;
-  const double rt = dot(r, F.t);
-  V3 rho = v3(rt * F.t.x - r.x, rt * F.t.y - r.y, rt * F.t.z - r.z);
-  const double rho2 = dot(rho, rho);
+  const double rt = TZ ? r.z : dot(r, F.t);
+  V3 rho = TZ ? v3(-r.x, -r.y, 0.0) : v3(rt * F.t.x - r.x, rt * F.t.y - r.y, rt * F.t.z - r.z);
+  const double rho2 = TZ ? r.x * r.x + r.y * r.y : dot(rho, rho);
   double LA = -box.hl - rt, LB = box.hl - rt;
   const double RA2 = LA * LA + rho2, RB2 = LB * LB + rho2;
   const double rsA = rsqrt(RA2), rsB = rsqrt(RB2);
@@ -88,7 +90,7 @@ __device__ __forceinline__ void box_add(const Fields<NF> &F, V3 r, const Box &bo
     LB = -LB;
     lA = -lA;
     lB = -lB;
-    rho = (-1.0) * rho;
+    rho = v3(-rho.x, -rho.y, TZ ? 0.0 : -rho.z);
   }
   // q = L + |R|; beside the segment (L < 0) the same as rho^2 / (|R| - L)
   double qA = fabs(LA) + RA2 * rsA, qB = fabs(LB) + RB2 * rsB;
@@ -106,6 +108,29 @@ __device__ __forceinline__ void box_add(const Fields<NF> &F, V3 r, const Box &bo
   const double h0 = 0.5 * d0, dt = h0 + d4;
   constexpr int IA[6] = {0, 1, 2, 0, 0, 1}, IC[6] = {0, 1, 2, 1, 2, 2};
   double T[6];             // the tensor of the beta term, shared by the fields
+  if constexpr (TZ) {
+    const double px = d2 * rho.x, py = d2 * rho.y;
+    T[0] = fma(rho.x, px, h0);
+    T[1] = fma(rho.y, py, h0);
+    T[2] = h0 + dt;
+    T[3] = rho.x * py;
+    T[4] = rho.x * d3;
+    T[5] = rho.y * d3;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const V3 b = F.b[f], w = F.w[f];                     // w = (b_y, -b_x, 0)
+      const double kb = F.k1 * (w.x * rho.x + w.y * rho.y);
+      const double cw = 0.5 * d1 * (1.0 - F.k1), hz = h0 * b.z;
+      const double yx = -h0 * F.k1 * rho.x, yy = -h0 * F.k1 * rho.y;
+      acc[f][0] += kb * T[0] + 2.0 * (w.x * yx);
+      acc[f][1] += kb * T[1] + 2.0 * (w.y * yy);
+      acc[f][2] += kb * T[2] + 2.0 * (h0 * (b.x * rho.y - b.y * rho.x));
+      acc[f][3] += kb * T[3] + (w.x * yy + w.y * yx);
+      acc[f][4] += kb * T[4] + (cw * w.x - hz * rho.y);
+      acc[f][5] += kb * T[5] + (cw * w.y + hz * rho.x);
+    }
+    return;
+  }
   const V3 p = d2 * rho + d3 * F.t, z = d3 * rho + dt * F.t;     // rho (d2 rho + d3 t) + t (d3 rho + dt t)
 #pragma unroll
   for (int c = 0; c < 6; ++c)
@@ -138,8 +163,8 @@ __device__ __forceinline__ int near_terms(const CoefGeom &g) {
 
 // Near-field coefficient: adds the term of subcell difference index q of the (2m-1)^3
 // lattice, times its multiplicity over the number of subcells.
-template <int NF>
-__device__ __forceinline__ void near_add(const CoefGeom &g, const Fields<NF> &F, V3 base, int q, double weight,
+template <int NF, bool TZ>
+__device__ __forceinline__ void near_add(const CoefGeom &g, const Fields<NF, TZ> &F, V3 base, int q, double weight,
                                          double (&acc)[NF][6]) {
   const int Dx = 2 * g.m[0] - 1, Dy = 2 * g.m[1] - 1;
   const int dx = q % Dx - (g.m[0] - 1);
@@ -147,12 +172,14 @@ __device__ __forceinline__ void near_add(const CoefGeom &g, const Fields<NF> &F,
   const int dz = q / (Dx * Dy) - (g.m[2] - 1);
   const double mult = (double)((g.m[0] - abs(dx)) * (g.m[1] - abs(dy)) * (g.m[2] - abs(dz)));
   const V3 r = base + v3(dx * g.hs[0], dy * g.hs[1], dz * g.hs[2]);
-  box_add<NF>(F, r, F.sub, weight * mult / (double)(g.m[0] * g.m[1] * g.m[2]), acc);
+  box_add(F, r, F.sub, weight * mult / (double)(g.m[0] * g.m[1] * g.m[2]), acc);
 }
 
 // Near field: |(i dx, j dy, k dz)|^2 < rn2, as ((x*x + y*y) + z*z) in round-to-nearest
 // double without contraction (the same decision as the plain IEEE expression).
+// Cells beyond near_lim along an axis are far without the FP64 test.
 __device__ __forceinline__ bool near_dev(const CoefGeom &g, int i, int j, int k) {
+  if (abs(i) > g.near_lim[0] || abs(j) > g.near_lim[1] || abs(k) > g.near_lim[2]) return false;
   const double x = __dmul_rn((double)i, g.h[0]), y = __dmul_rn((double)j, g.h[1]), z = __dmul_rn((double)k, g.h[2]);
   return __dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z)) < g.rn2;
 }
@@ -179,8 +206,8 @@ __device__ __forceinline__ int min_images(int i, int n, int r[2], double w[2]) {
 // subcell differences of every near image together (one near image is up to a few
 // hundred terms), so they finish at about the same time.  Every lane of a warp calls
 // this with the same number of images; `lanes`: the warp's mask of this offset's lanes.
-template <int NF, int S>
-__device__ __forceinline__ void coef_share(const CoefGeom &g, const Fields<NF> &F, int i, int j, int k, int lane,
+template <int S, int NF, bool TZ>
+__device__ __forceinline__ void coef_share(const CoefGeom &g, const Fields<NF, TZ> &F, int i, int j, int k, int lane,
                                            unsigned lanes, double (&acc)[NF][6]) {
   const int n = g.n_shells, side = 2 * n + 1, images = side * side;
   int rx[2] = {i, 0}, ry[2] = {j, 0};
@@ -198,25 +225,26 @@ __device__ __forceinline__ void coef_share(const CoefGeom &g, const Fields<NF> &
         const int m = m0 + lane;
         const int ii = rx[a] + (m / side - n) * g.nx, jj = ry[b] + (m % side - n) * g.ny;
         const bool near = m < images && near_dev(g, ii, jj, k);
-        if (m < images && !near) box_add<NF>(F, offset_pos(g, ii, jj, k), F.cell, wt, acc);
+        if (m < images && !near) box_add(F, offset_pos(g, ii, jj, k), F.cell, wt, acc);
         unsigned mask = S > 1 ? __ballot_sync(lanes, near) & lanes : (near ? 1u : 0u);
         while (mask) {                        // this offset's near images, all its lanes on each
           const int bit = __ffs(mask) - 1;
           mask &= mask - 1;
           const int q = m0 + (S > 1 ? bit % S : 0);
           const V3 base = offset_pos(g, rx[a] + (q / side - n) * g.nx, ry[b] + (q % side - n) * g.ny, k);
-          for (int d = lane; d < terms; d += S) near_add<NF>(g, F, base, d, wt, acc);
+          for (int d = lane; d < terms; d += S) near_add(g, F, base, d, wt, acc);
         }
       }
     }
 }
 
 // ---- coefficients at listed offsets (parity queries) ------------------------
-__global__ void k_table_at(CoefGeom g, Fields<1> F, long n, const int *ijk, double *out) {
+template <bool TZ>
+__global__ void k_table_at(CoefGeom g, Fields<1, TZ> F, long n, const int *ijk, double *out) {
   const long q = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (q >= n) return;
   double acc[1][6] = {{0, 0, 0, 0, 0, 0}};
-  coef_share<1, 1>(g, F, ijk[3 * q], ijk[3 * q + 1], ijk[3 * q + 2], 0, 0u, acc);
+  coef_share<1>(g, F, ijk[3 * q], ijk[3 * q + 1], ijk[3 * q + 2], 0, 0u, acc);
 #pragma unroll
   for (int c = 0; c < 6; ++c) out[6 * q + c] = acc[0][c];
 }
@@ -233,14 +261,14 @@ struct Tab {
 __host__ __device__ __forceinline__ long tab_size(const Tab &T) { return (long)T.nz * T.ry * T.rx; }
 
 // One segment per offset (near offsets are overwritten by k_table_near).
-template <int NF>
-__global__ void __launch_bounds__(256) k_table_far(CoefGeom g, Fields<NF> F, Tab T, double *tab) {
+template <int NF, bool TZ>
+__global__ void __launch_bounds__(256) k_table_far(CoefGeom g, Fields<NF, TZ> F, Tab T, double *tab) {
   const long N = tab_size(T), idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (idx >= N) return;
   const int ir = (int)(idx % T.rx), jr = (int)((idx / T.rx) % T.ry), k = (int)(idx / ((long)T.rx * T.ry));
   const int i = ir < T.nx ? ir : ir - (2 * T.nx - 1), j = jr < T.ny ? jr : jr - (2 * T.ny - 1);
   double acc[NF][6] = {};
-  box_add<NF>(F, offset_pos(g, i, j, k), F.cell, 1.0, acc);
+  box_add(F, offset_pos(g, i, j, k), F.cell, 1.0, acc);
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
@@ -248,8 +276,8 @@ __global__ void __launch_bounds__(256) k_table_far(CoefGeom g, Fields<NF> F, Tab
 }
 
 // Replica sums: S lanes per offset.
-template <int NF, int S>
-__global__ void __launch_bounds__(256) k_table_pbc(CoefGeom g, Fields<NF> F, Tab T, double *tab) {
+template <int NF, bool TZ, int S>
+__global__ void __launch_bounds__(256) k_table_pbc(CoefGeom g, Fields<NF, TZ> F, Tab T, double *tab) {
   const long N = tab_size(T), idx = (blockIdx.x * (long)blockDim.x + threadIdx.x) / S;
   if (idx >= N) return;                       // all lanes of an offset together
   const int lane = threadIdx.x % S;
@@ -257,7 +285,7 @@ __global__ void __launch_bounds__(256) k_table_pbc(CoefGeom g, Fields<NF> F, Tab
   const int ir = (int)(idx % T.rx), jr = (int)((idx / T.rx) % T.ry), k = (int)(idx / ((long)T.rx * T.ry));
   const int i = ir < T.nx ? ir : ir - (2 * T.nx - 1), j = jr < T.ny ? jr : jr - (2 * T.ny - 1);
   double acc[NF][6] = {};
-  coef_share<NF, S>(g, F, i, j, k, lane, lanes, acc);
+  coef_share<S>(g, F, i, j, k, lane, lanes, acc);
 #pragma unroll
   for (int f = 0; f < NF; ++f)
 #pragma unroll
@@ -269,14 +297,14 @@ __global__ void __launch_bounds__(256) k_table_pbc(CoefGeom g, Fields<NF> F, Tab
 }
 
 // One block per near offset (rows of the table): reduce the subcell-difference lattice.
-template <int NF>
-__global__ void __launch_bounds__(128) k_table_near(CoefGeom g, Fields<NF> F, Tab T, const int *ijk, double *tab) {
+template <int NF, bool TZ>
+__global__ void __launch_bounds__(128) k_table_near(CoefGeom g, Fields<NF, TZ> F, Tab T, const int *ijk, double *tab) {
   const int q = blockIdx.x;
   const int i = ijk[3 * q], j = ijk[3 * q + 1], k = ijk[3 * q + 2];
   const V3 base = offset_pos(g, i, j, k);
   double acc[NF][6] = {};
   const int terms = near_terms(g);
-  for (int d = threadIdx.x; d < terms; d += blockDim.x) near_add<NF>(g, F, base, d, 1.0, acc);
+  for (int d = threadIdx.x; d < terms; d += blockDim.x) near_add(g, F, base, d, 1.0, acc);
   __shared__ double red[4][NF * 6];
 #pragma unroll
   for (int f = 0; f < NF; ++f)
@@ -558,19 +586,18 @@ __global__ void k_extract_four(const double *spec, int fold, Shape sh, int e, in
                                const unsigned long long *amax, OT *kspec) {
   constexpr int V = 16 / (int)sizeof(OT);
   const int W = sh.wz, R2 = zfour_r2(sh.pz), R1 = sh.pz / R2, M = sh.M, py = sh.py, fe = sh.fe;
-  const long per_tile = (long)sh.pz * W;
-  const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  if (idx >= zf_stored_tiles(sh) * per_tile) return;
-  const long s = idx / per_tile;
-  const int r = (int)(idx - s * per_tile), t = r / R2, k2 = r % R2, k1 = t / W, w = t % W, q = R2 * e + k2;
-  const long ktiles = M / W;
-  const long main_tiles = (long)(sh.zs.xall ? py / 2 + 1 : py) * ktiles;
+  // 32-bit indices: at most 1024 x 513 x 512 values
+  const unsigned per_tile = sh.pz * W, idx = blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (unsigned)zf_stored_tiles(sh) * per_tile) return;
+  const int s = idx / per_tile, r = idx - s * per_tile, t = r / R2, k2 = r % R2, k1 = t / W, w = t % W, q = R2 * e + k2;
+  const int ktiles = M / W;
+  const int main_tiles = (sh.zs.xall ? py / 2 + 1 : py) * ktiles;
   int kx, ky;
   if (s < main_tiles) {
-    ky = (int)(s / ktiles);
-    kx = (int)(s % ktiles) * W + w;
+    ky = s / ktiles;
+    kx = (s - ky * ktiles) * W + w;
   } else {
-    ky = (int)(s - main_tiles) * W + w;
+    ky = (s - main_tiles) * W + w;
     kx = M;
   }
   double v = spec_at(spec, M, py, sh.pz, fold, kx, ky, k1 + R1 * k2) * scale;
@@ -578,7 +605,7 @@ __global__ void k_extract_four(const double *spec, int fold, Shape sh, int e, in
     const double m = __longlong_as_double((long long)*amax) * scale;
     if (m > 0.0) v /= m;
   }
-  const size_t dst = (size_t)(s * 6 + c) * fe * per_tile + ((size_t)(q / V) * (R1 * W) + t) * V + q % V;
+  const size_t dst = ((size_t)s * 6 + c) * fe * per_tile + ((size_t)(q / V) * (R1 * W) + t) * V + q % V;
   store_val(&kspec[dst], v);
 }
 
@@ -670,6 +697,8 @@ CoefGeom coef_geom(const dds_ctx *ctx) {
   const double hmax = fmax(ctx->h[0], fmax(ctx->h[1], ctx->h[2]));
   const double rn = ctx->n_near * hmax;
   g.rn2 = rn * rn;
+  // |i| h < rn in exact arithmetic, with a cell to spare for rounding
+  for (int a = 0; a < 3; ++a) g.near_lim[a] = (int)fmin(1e9, ceil(rn / ctx->h[a]) + 1.0);
   g.nx = ctx->nx;
   g.ny = ctx->ny;
   g.n_shells = ctx->n_shells;
@@ -688,9 +717,9 @@ Box make_box(const double hb[3], const double t[3], double mu) {
 }
 
 // Fields of one line direction (nf <= NF of them; the rest repeat the last).
-template <int NF>
-Fields<NF> make_fields(const CoefGeom &g, const double t[3], const double *b) {
-  Fields<NF> F;
+template <int NF, bool TZ>
+Fields<NF, TZ> make_fields(const CoefGeom &g, const double t[3], const double *b) {
+  Fields<NF, TZ> F;
   F.t = v3(t[0], t[1], t[2]);
   for (int f = 0; f < NF; ++f) {
     const double *q = b + 3 * f;
@@ -704,23 +733,32 @@ Fields<NF> make_fields(const CoefGeom &g, const double t[3], const double *b) {
 }
 
 // Table of NF fields (near: the stored near offsets, open boundary only).
-template <int NF>
-cudaError_t fill_table(const CoefGeom &g, const double t[3], const double *b, const Tab &T, int n_near,
+template <int NF, bool TZ>
+cudaError_t fill_table_dir(const CoefGeom &g, const double t[3], const double *b, const Tab &T, int n_near,
                        const int *d_near, double *tab, cudaStream_t s) {
-  const Fields<NF> F = make_fields<NF>(g, t, b);
+  const Fields<NF, TZ> F = make_fields<NF, TZ>(g, t, b);
   const long N = tab_size(T);
   if (g.n_shells > 2)                         // 49 images and more: a warp per offset
-    k_table_pbc<NF, 32><<<(unsigned)((N * 32 + 255) / 256), 256, 0, s>>>(g, F, T, tab);
+    k_table_pbc<NF, TZ, 32><<<(unsigned)((N * 32 + 255) / 256), 256, 0, s>>>(g, F, T, tab);
   else if (g.n_shells > 0)                    // 9 or 25 images
-    k_table_pbc<NF, 8><<<(unsigned)((N * 8 + 255) / 256), 256, 0, s>>>(g, F, T, tab);
+    k_table_pbc<NF, TZ, 8><<<(unsigned)((N * 8 + 255) / 256), 256, 0, s>>>(g, F, T, tab);
   else
-    k_table_far<NF><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(g, F, T, tab);
+    k_table_far<NF, TZ><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(g, F, T, tab);
   cudaError_t err = cudaGetLastError();
   if (err == cudaSuccess && n_near > 0) {
-    k_table_near<NF><<<n_near, 128, 0, s>>>(g, F, T, d_near, tab);
+    k_table_near<NF, TZ><<<n_near, 128, 0, s>>>(g, F, T, d_near, tab);
     err = cudaGetLastError();
   }
   return err;
+}
+
+bool vertical(const double t[3]) { return t[0] == 0.0 && t[1] == 0.0 && t[2] == 1.0; }
+
+template <int NF>
+cudaError_t fill_table(const CoefGeom &g, const double t[3], const double *b, const Tab &T, int n_near,
+                       const int *d_near, double *tab, cudaStream_t s) {
+  return vertical(t) ? fill_table_dir<NF, true>(g, t, b, T, n_near, d_near, tab, s)
+                     : fill_table_dir<NF, false>(g, t, b, T, n_near, d_near, tab, s);
 }
 
 // Consecutive effective fields whose tables are made together.
@@ -735,7 +773,9 @@ cudaError_t launch_table_at(const CoefGeom &g, const double t[3], const double b
                             const int *d_ijk, double *d_out, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int nt = 128;
-  k_table_at<<<(unsigned)((n + nt - 1) / nt), nt, 0, s>>>(g, make_fields<1>(g, t, b), n, d_ijk, d_out);
+  const unsigned blocks = (unsigned)((n + nt - 1) / nt);
+  if (vertical(t)) k_table_at<true><<<blocks, nt, 0, s>>>(g, make_fields<1, true>(g, t, b), n, d_ijk, d_out);
+  else k_table_at<false><<<blocks, nt, 0, s>>>(g, make_fields<1, false>(g, t, b), n, d_ijk, d_out);
   return cudaGetLastError();
 }
 

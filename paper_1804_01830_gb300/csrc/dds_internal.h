@@ -88,6 +88,7 @@ struct CoefGeom {
   int m[3];           // subcells per axis
   double mu, nu;
   double rn2;         // squared near-field radius (n_near * max h)^2
+  int near_lim[3];    // no near cell lies farther than this many cells along an axis
   int nx, ny;         // grid (replica periods)
   int n_shells;       // > 0: replica shells of the in-plane periodic boundary conditions
   int periodic;       // with n_shells > 0: shells centred on each source's minimal image
