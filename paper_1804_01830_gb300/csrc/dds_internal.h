@@ -52,9 +52,9 @@ struct Shape {
   // zfour: after the forward y pass the main array is [ky][z tile][field][z][column of the
   // tile] instead of [field][z][ky][kx], so that a z tile reads one contiguous block: its
   // 64-byte row pieces otherwise lie a plane apart, one to a DRAM page (GaN layer, z pass 0.92
-  // -> 0.82 ms for 0.03 ms more in the y pass; 90x77x200 0.41 -> 0.36 ms).  Not for 1024 rows,
-  // whose y tiles are four columns wide: 32-byte writes cost the y pass more (512x512x64, two
-  // sets, 0.90 -> 1.35 ms) than the z pass gains.
+  // -> 0.82 ms for 0.03 ms more in the y pass; 90x77x200 0.41 -> 0.36 ms).  Not for 1024 rows:
+  // there the y pass loses more (512x512x64, two sets, 0.75 -> 0.89 ms) than the z pass gains
+  // (3.07 -> 3.01 ms).
   int ztile;
   int nb;             // density sets evaluated together (batch); fields are [b][e], outputs [b][c]
   ZSym zs;            // zfour: stored-spectrum symmetries and layout

@@ -81,79 +81,6 @@ cudaError_t persistent_grid(int threads, size_t smem, long tiles, const DevInfo 
   return cudaSuccess;
 }
 
-// ------------------------------------------------------------- y passes -----
-// Forward: rows y < ny in, all py rows out.  Inverse: all py rows in, y < ny out.
-template <int PY, int W, int NT, bool INV>
-__global__ void __launch_bounds__(NT) k_ypass(Shape sh, int nf, const float2 *in_main, const float2 *in_nyq,
-                                              float2 *out_main, float2 *out_nyq, const float2 *tw) {
-  constexpr int LD = W, PB = Plan<PY>::r0;
-  extern __shared__ float2 smem[];
-  float2 *buf = smem;
-  pdl_trigger();
-  pdl_wait();
-  const int tid = threadIdx.x;
-  const int M = sh.M, nz = sh.nz;
-  const int rows_in = INV ? PY : sh.ny;
-  const int rows_out = INV ? sh.ny : PY;
-  const long ktiles = M / W;
-  const long tiles_main = (long)nf * nz * ktiles;
-  const long tau = blockIdx.x;
-  const float2 *in;
-  float2 *out;
-  long rs;
-  int ncols;
-  if (tau < tiles_main) {
-    const int e = (int)(tau / (nz * ktiles));
-    const long r = tau - (long)e * nz * ktiles;
-    const int z = (int)(r / ktiles), kt = (int)(r - (long)z * ktiles);
-    in = in_main + ((long)(e * nz + z) * rows_in) * M + kt * W;
-    out = out_main + ((long)(e * nz + z) * rows_out) * M + kt * W;
-    rs = M;
-    ncols = W;
-  } else {
-    const long t2 = tau - tiles_main;
-    const int ztiles = (nz + W - 1) / W;
-    const int e = (int)(t2 / ztiles), zt = (int)(t2 - (long)e * ztiles);
-    in = in_nyq + (long)e * rows_in * nz + zt * W;
-    out = out_nyq + (long)e * rows_out * nz + zt * W;
-    rs = nz;
-    ncols = min(W, nz - zt * W);
-  }
-  if (tau < tiles_main) {            // rows of W complex, 16-byte aligned: 16-byte copies
-    constexpr int H = W / 2;
-    for (int p = tid; p < rows_in * H; p += NT) {
-      const int n = p / H, c2 = p - n * H;
-      cp_async16(&buf[tidx<LD, PB, W>(n, 2 * c2)], &in[n * rs + 2 * c2]);
-    }
-  } else {
-    for (int p = tid; p < rows_in * W; p += NT) {
-      const int n = p / W, w = p - n * W;
-      if (w < ncols) cp_async8(&buf[tidx<LD, PB, W>(n, w)], &in[n * rs + w]);
-      else buf[tidx<LD, PB, W>(n, w)] = make_float2(0.f, 0.f);
-    }
-  }
-  if (!INV) {
-    for (int p = rows_in * W + tid; p < (PY / 2) * W; p += NT) buf[tidx<LD, PB, W>(p / W, p % W)] = make_float2(0.f, 0.f);
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  fft_tile<PY, W, LD, NT, INV, !INV, INV, PB>(buf, tw + tw_offset(PY), tid);
-  if (tau < tiles_main) {            // 16-byte stores of column pairs
-    constexpr int H = W / 2;
-    for (int p = tid; p < rows_out * H; p += NT) {
-      const int n = p / H, c2 = p - n * H;
-      *reinterpret_cast<float4 *>(&out[n * rs + 2 * c2]) =
-          *reinterpret_cast<const float4 *>(&buf[tidx<LD, PB, W>(n, 2 * c2)]);
-    }
-  } else {
-    for (int p = tid; p < rows_out * W; p += NT) {
-      const int n = p / W, w = p - n * W;
-      if (w < ncols) out[n * rs + w] = buf[tidx<LD, PB, W>(n, w)];
-    }
-  }
-}
-
-
 // s = sqrt(sum / (nx ny)) for every (set, component, height).
 __global__ void k_stats_finish(const double *sums, long n, double inv_plane, float *s_out) {
   pdl_trigger();
@@ -210,13 +137,6 @@ cudaError_t launch_y(const Shape &sh, int nf, const float2 *im, const float2 *in
       return launch_pass<yr::k_ypass_st<PY, W, T, INV, true>>(sh.early, (unsigned)tiles, T, smem, s, sh, nf, im, in, om, on, tw);
     }
     return cudaErrorInvalidValue;
-  }
-  if constexpr (INV && PY >= 1024) {
-    // 1024-row inverse: the shared-memory Stockham tile with 16-byte row stores (radial
-    // disk 512x512x16: 0.137 ms, against 0.152 for the register stages on 4-column
-    // tiles and 0.146 on 8-column tiles of 256 threads)
-    const size_t smem = sizeof(float2) * tile_elems<PY, W, Plan<PY>::r0, W>();
-    return launch_pass<k_ypass<PY, W, T, INV>>(sh.early, (unsigned)tiles, T, smem, s, sh, nf, im, in, om, on, tw);
   }
   const size_t smem = sizeof(float2) * yr::y_smem_all<PY, W, INV, false>();
   return launch_pass<yr::k_ypass_st<PY, W, T, INV, false>>(sh.early, (unsigned)tiles, T, smem, s, sh, nf, im, in, om, on, tw);

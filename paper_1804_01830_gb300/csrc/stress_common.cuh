@@ -12,15 +12,17 @@ namespace dds {
 
 constexpr int NT = 256;   // threads of the shared-memory z pass
 
-// Tile shape of the y passes: W columns per tile, NT threads.  Small tiles keep
-// several CTAs resident per SM so that one tile's copies overlap another tile's
-// transform.
+// Small y tiles keep several CTAs resident per SM, so that one tile's copies overlap another
+// tile's transform.
 // y-pass tiles: W columns, NT threads.  The 512-row inverse takes 16 columns and 256
 // threads (whole 128-byte rows; GaN layer 0.215 -> 0.207 ms); the 512-row forward keeps
-// 8 and 128 (0.176 against 0.183 ms with 16).
+// 8 and 128 (0.176 against 0.183 ms with 16).  1024 rows take 8 columns and 256 threads in
+// both directions, in register stages like the others (512x512x64, two sets, against 4
+// columns: forward 0.84 -> 0.75 ms; inverse, there in a shared-memory Stockham tile, 0.96 ->
+// 0.84 ms; radial disk inverse 0.131 -> 0.119 ms).
 template <int P, bool INV = false> struct YTile {
-  static constexpr int W = P >= 1024 ? 4 : (P >= 512 ? (INV ? 16 : 8) : 16);
-  static constexpr int NT = (P == 512 && INV) ? 256 : 128;
+  static constexpr int W = P >= 1024 ? 8 : (P >= 512 ? (INV ? 16 : 8) : 16);
+  static constexpr int NT = (P == 1024 || (P == 512 && INV)) ? 256 : 128;
 };
 
 __device__ __forceinline__ float2 cmadd_i(float2 acc, float g, float2 r) {
