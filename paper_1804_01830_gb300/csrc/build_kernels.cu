@@ -789,9 +789,9 @@ int build_spectra(dds_ctx *ctx, cudaStream_t s) {
   const double *ft = ctx->field_t.data(), *fb = ctx->field_b.data();
 
   // workspace: at most what a full padded FP64 table of one field and one complex
-  // spectrum take (or 1 GB): fields of one direction share a table, and as many
-  // components as fit share a launch
-  const size_t limit = std::max((size_t)1 << 30, 48 * P + 16 * (size_t)(M + 1) * py * pz);
+  // spectrum take: fields of one direction share a table, and as many components as fit
+  // share a launch
+  const size_t limit = 48 * P + 16 * (size_t)(M + 1) * py * pz;
   auto tab_of = [&](int mx, int my) {
     Tab T;
     T.nx = sh.nx;
@@ -825,7 +825,7 @@ int build_spectra(dds_ctx *ctx, cudaStream_t s) {
     const int least = b.mx ? 2 : 1;
     int slots = 6;
     auto total = [&]() { return 48 * (size_t)b.n * tab_size(T) + slots * (std::max(x, z) + y); };
-    while (total() > limit && slots > least) slots = slots > 2 ? 2 : least;
+    while (total() > limit && slots > least) slots = slots > 2 ? slots - 2 : least;
     while (total() > limit && b.n > 1) --b.n;
     batches.push_back(b);
     slots_of.push_back(slots);
