@@ -112,6 +112,9 @@ cudaError_t launch_x_fwd(const Shape &sh, const Collapse &col, const void *rho, 
     GroupList &gl = d ? direct : accum;
     gl.g[gl.n++] = g;
   }
+  // groups with more families first: their CTAs run longer, and the short ones fill the last
+  // wave (x forward: GaN layer 0.201 -> 0.197 ms, BF16 batch of 128^3 0.193 -> 0.187 ms)
+  std::stable_sort(accum.g, accum.g + accum.n, [&](int a, int b) { return col.nf[a] > col.nf[b]; });
   cudaError_t err = cudaSuccess;
   if (direct.n > 0) {
     err = bf16 ? launch_x_fwd_kind<M, true, true>(sh, col, direct, rho, om, on, tw, s)
