@@ -339,7 +339,11 @@ k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v
       for (int n1 = 0; n1 < H; ++n1) acc[d][q][n1] = make_float2(0.f, 0.f);
   const int nfam = DIRECT ? 1 : col.nf[g];
   if (live) {
-#pragma unroll 2
+    // one family at a time, all its loads in flight: two cost registers that the later stages
+    // lack (GaN layer 0.197 -> 0.194 ms, 256x256x64 in BF16 0.104 -> 0.088 ms), except for short
+    // BF16 rows read value by value (101x90x77: 0.058 against 0.062 ms)
+    constexpr int UNROLL = BF16 && !WIDE && M <= 128 ? 2 : 1;
+#pragma unroll UNROLL
     for (int f = 0; f < nfam; ++f) {
       const int fi = col.f0[g] + f;
       const long base = set_off + (long)col.fam[fi] * N + line * sh.nx;
