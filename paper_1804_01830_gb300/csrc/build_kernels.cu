@@ -761,9 +761,9 @@ cudaError_t fill_table(const CoefGeom &g, const double t[3], const double *b, co
                      : fill_table_dir<NF, false>(g, t, b, T, n_near, d_near, tab, s);
 }
 
-// Consecutive effective fields whose tables are made together.
+// Consecutive effective fields whose tables are made together; components per launch.
 struct Batch {
-  int e0, n, mx, my;
+  int e0, n, mx, my, slots;
 };
 
 }  // namespace
@@ -788,10 +788,6 @@ int build_spectra(dds_ctx *ctx, cudaStream_t s) {
   const CoefGeom g = coef_geom(ctx);
   const double *ft = ctx->field_t.data(), *fb = ctx->field_b.data();
 
-  // workspace: at most what a full padded FP64 table of one field and one complex
-  // spectrum take: fields of one direction share a table, and as many components as fit
-  // share a launch
-  const size_t limit = 48 * P + 16 * (size_t)(M + 1) * py * pz;
   auto tab_of = [&](int mx, int my) {
     Tab T;
     T.nx = sh.nx;
@@ -803,37 +799,56 @@ int build_spectra(dds_ctx *ctx, cudaStream_t s) {
     T.ry = (my || py == sh.ny) ? sh.ny : 2 * sh.ny - 1;      // periodic in y: rows 0 .. ny - 1
     return T;
   };
-  auto slot_bytes = [&](const Tab &T, size_t *x, size_t *y, size_t *z) {
-    const size_t ky = T.mx ? py / 2 + 1 : py, c = M + 1;
-    *x = (size_t)T.nz * T.ry * c * (T.mx ? 8 : 16);
-    *y = (size_t)T.nz * ky * c * 16;
-    *z = (size_t)pz * ky * c * 8;
+  // Runs of up to three fields of one direction and mirrors share tables, and up to six
+  // components share a launch.  The three buffers are each sized for the run that needs most
+  // of it; their sum is kept within what a full padded FP64 table of one field and one complex
+  // spectrum take (sized run by run without that rule, 18 families on 256x256x128 took 4.03 GB
+  // against 3.76, a mirrored and an unmirrored direction together 4.83).  Components per launch
+  // are reduced first, where they take most, then fields per table.  The fewest of both always
+  // fit: half of that table, and half of that spectrum in each buffer.
+  struct Run {
+    int e0, fields, mx, my;
+    int n, slots;               // fields per table, components per launch
+    size_t tab, x, y;           // bytes per field of a table, per component of either buffer
+    int least() const { return mx ? 2 : 1; }
   };
-  std::vector<Batch> batches;
-  size_t tab_max = 0, buf1_max = 0, buf2_max = 0;
-  std::vector<int> slots_of;
+  std::vector<Run> runs;
   for (int e = 0; e < ctx->fe;) {
     auto flag = [&](int q, int a) { return mirror_ok(ft + 3 * q, fb + 3 * q, a) ? 1 : 0; };
-    Batch b{e, 1, flag(e, 0), flag(e, 1)};
-    while (b.n < 3 && e + b.n < ctx->fe && flag(e + b.n, 0) == b.mx && flag(e + b.n, 1) == b.my &&
-           ft[3 * e] == ft[3 * (e + b.n)] && ft[3 * e + 1] == ft[3 * (e + b.n) + 1] &&
-           ft[3 * e + 2] == ft[3 * (e + b.n) + 2])
-      ++b.n;
-    const Tab T = tab_of(b.mx, b.my);
-    size_t x, y, z;
-    slot_bytes(T, &x, &y, &z);
-    const int least = b.mx ? 2 : 1;
-    int slots = 6;
-    auto total = [&]() { return 48 * (size_t)b.n * tab_size(T) + slots * (std::max(x, z) + y); };
-    while (total() > limit && slots > least) slots = slots > 2 ? slots - 2 : least;
-    while (total() > limit && b.n > 1) --b.n;
-    batches.push_back(b);
-    slots_of.push_back(slots);
-    tab_max = std::max(tab_max, 48 * (size_t)b.n * tab_size(T));
-    buf1_max = std::max(buf1_max, slots * std::max(x, z));
-    buf2_max = std::max(buf2_max, slots * y);
-    e += b.n;
+    Run r{e, 1, flag(e, 0), flag(e, 1), 0, 6, 0, 0, 0};
+    while (r.fields < 3 && e + r.fields < ctx->fe && flag(e + r.fields, 0) == r.mx && flag(e + r.fields, 1) == r.my &&
+           ft[3 * e] == ft[3 * (e + r.fields)] && ft[3 * e + 1] == ft[3 * (e + r.fields) + 1] &&
+           ft[3 * e + 2] == ft[3 * (e + r.fields) + 2])
+      ++r.fields;
+    const Tab T = tab_of(r.mx, r.my);
+    const size_t ky = T.mx ? py / 2 + 1 : py, c = M + 1;
+    r.n = r.fields;
+    r.tab = 48 * (size_t)tab_size(T);
+    r.x = std::max((size_t)T.nz * T.ry * c * (T.mx ? 8 : 16), (size_t)pz * ky * c * 8);
+    r.y = (size_t)T.nz * ky * c * 16;
+    runs.push_back(r);
+    e += r.fields;
   }
+  size_t tab_max = 0, buf1_max = 0, buf2_max = 0;
+  const size_t limit = 48 * P + 16 * (size_t)(M + 1) * py * pz;
+  for (;;) {
+    tab_max = buf1_max = buf2_max = 0;
+    Run *wide = nullptr, *deep = nullptr;     // most in the buffers and reducible; largest table
+    for (Run &r : runs) {
+      tab_max = std::max(tab_max, r.n * r.tab);
+      buf1_max = std::max(buf1_max, r.slots * r.x);
+      buf2_max = std::max(buf2_max, r.slots * r.y);
+      if (r.slots > r.least() && (!wide || r.slots * (r.x + r.y) > wide->slots * (wide->x + wide->y))) wide = &r;
+      if (r.n > 1 && (!deep || r.n * r.tab > deep->n * deep->tab)) deep = &r;
+    }
+    if (tab_max + buf1_max + buf2_max <= limit) break;
+    if (wide) wide->slots = wide->slots > 2 ? wide->slots - 2 : wide->least();
+    else if (deep) --deep->n;
+    else break;
+  }
+  std::vector<Batch> batches;
+  for (const Run &r : runs)
+    for (int f = 0; f < r.fields; f += r.n) batches.push_back({r.e0 + f, std::min(r.n, r.fields - f), r.mx, r.my, r.slots});
 
   // near offsets the tables hold (decided on the host, same expression as the
   // definition): all of them, then those with i >= 0, j >= 0 and both, by (mx, my)
@@ -917,7 +932,7 @@ int build_spectra(dds_ctx *ctx, cudaStream_t s) {
         Comps C = all;
         for (; q < sets.size(); ++q) {
           const int add = sets[q].second >= 0 ? 2 : 1;
-          if (C.slots + add > slots_of[ib]) break;
+          if (C.slots + add > b.slots) break;
           C.ce[C.sets] = sets[q].first;
           C.co[C.sets] = sets[q].second;
           C.se[C.sets] = C.slots;
