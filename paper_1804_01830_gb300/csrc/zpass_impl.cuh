@@ -264,10 +264,22 @@ template <int E> struct GRaw<__half, E> {
   }
 };
 
+// CTAs per SM k_zreg is compiled for.  The compiler left alone takes a register or two more
+// than one more CTA allows (padded z 64, FP16 spectra, four fields: 158, three CTAs): at four
+// CTAs and 128 registers, without spills, 100x100x32 185 -> 161 us an evaluation, 256x128x32
+// 362 -> 298; two fields, FP32, at five CTAs 110 -> 98 and 203 -> 189.  The single field on
+// two lanes is faster left alone (256x256x16, FP32: 114 against 117 us).
+template <int E, int G, int FE, typename GT> constexpr int zreg_ctas() {
+  constexpr bool half = sizeof(GT) == 2;
+  if (E == 8) return FE == 1 ? 6 : (FE == 2 ? 5 : (G == 8 && half ? 4 : 3));
+  if (FE == 1) return G == 2 ? 1 : (G == 1 && half ? 5 : 4);
+  return FE == 2 && half ? 3 : 2;
+}
+
 template <int E, int G, int FE, typename GT>
-__global__ void __launch_bounds__(128) k_zreg(Shape sh, const float2 *in_main, const float2 *in_nyq,
-                                              const GT *kspec, const float *kscale, float2 *out_main,
-                                              float2 *out_nyq, const float2 *tw) {
+__global__ void __launch_bounds__(128, (zreg_ctas<E, G, FE, GT>()))
+    k_zreg(Shape sh, const float2 *in_main, const float2 *in_nyq, const GT *kspec, const float *kscale,
+           float2 *out_main, float2 *out_nyq, const float2 *tw) {
   constexpr int P = G * E, CW = 32 / G;
   pdl_trigger();
   pdl_wait();
@@ -297,8 +309,11 @@ __global__ void __launch_bounds__(128) k_zreg(Shape sh, const float2 *in_main, c
   const float2 *twP = tw + tw_offset(P);
 
   // rows z of this lane's column in the inputs and outputs: one pointer and stride for
-  // both kinds of tile, so that all loads are in flight together
-  const long sz = nyq ? 1 : (long)py * M, se = (long)nz * py * (nyq ? 1 : M);
+  // both kinds of tile, so that all loads are in flight together.  A set is at most
+  // 6 x 32 x 1024 x 512 values: 32-bit strides save the registers that a further CTA needs
+  // (the single field on one or two lanes takes fewer with 64-bit ones)
+  using Stride = std::conditional_t<FE == 1 && G <= 2, long, int>;
+  const Stride sz = nyq ? 1 : (Stride)py * M, se = (Stride)nz * py * (nyq ? 1 : M);
   const float2 *src = nyq ? in_nyq + ky * nz : in_main + ky * M + kx;
   float2 *dst = nyq ? out_nyq + ky * nz : out_main + ky * M + kx;
   float2 f[FE][E];
