@@ -63,11 +63,12 @@ enum {
   DDS_OPT_Z_LANES = 2,     /* schedule of the fused z pass: 0 = automatic (default);
                               -1 = shared-memory tiles; -2 = three-stage register kernel
                               (padded z size 128 or 256, <= 6 combined fields; the
-                              automatic choice there, and for padded z 512 up to 5 fields
-                              and 32 and 64 with 5 or 6); 1, 2, 4, 8 = register-only kernel
-                              with that many lanes per (kx, ky) column (needs padded
-                              z size <= 64 and <= 4 combined fields).  Same result up to
-                              rounding; a tuning knob.  A schedule the grid cannot take
+                              automatic choice there, for padded z 512 up to 5 fields, and
+                              for padded z 32 and 64 with 5 or 6 where nx > 16, at padded z
+                              64 or with 6 fields only from 100 tiles of 32 columns on);
+                              1, 2, 4, 8 = register-only kernel with that many lanes per
+                              (kx, ky) column (needs padded z size <= 64 and <= 4 combined
+                              fields).  Same result up to rounding; a tuning knob.  A schedule the grid cannot take
                               fails dds_build_kernels with DDS_ERR_UNSUPPORTED.
                               Invalidates built kernels. */
   DDS_OPT_PBC_SHELLS = 4,  /* in-plane periodic boundary conditions (Sec. 4): n > 0 makes

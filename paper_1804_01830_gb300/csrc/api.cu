@@ -268,14 +268,16 @@ int make_plan(dds_ctx *ctx) {
   // default there); by default also padded z 512 up to 5 fields (more than that has no
   // schedule there), and 32 and 64 where more than four fields rule out the register-only
   // pass: against shared-memory tiles, z pass of 90x77x200 (three fields) 0.81 -> 0.43 ms, of
-  // 250x241x29 (five fields, half the spectra) 0.37 -> 0.20 ms.  Padded z 64 with fewer than
-  // 100 tiles would leave most SMs idle: 30x30x30, 64 tiles, 18.4 against 16.3 us; 64x32x32,
-  // 128 tiles, 18.4 against 20.4 us.
+  // 250x241x29 (five fields, half the spectra) 0.37 -> 0.20 ms.  Padded z 64, or six fields,
+  // with fewer than 100 tiles would leave most SMs idle: padded z 64, 30x30x30, 64 tiles, 18.4
+  // against 16.3 us; 64x32x32, 128 tiles, 18.4 against 20.4 us; padded z 32 with six fields, an
+  // evaluation of 20x10x16, 32 tiles, 25.8 against 23.8 us; 30x40x10, 128 tiles, 26.8 against
+  // 29.3.  Five fields gain there from the smallest grid on (20x10x16 20.5 against 23.1).
   const int fw = zfour_width(sh.pz);
   const bool fits = sh.fe <= 6 && sh.M % fw == 0 && sh.py % fw == 0;
   const bool four_ok = (sh.pz == 128 || sh.pz == 256) && fits;
   const bool four_auto = four_ok || (fits && (sh.pz == 512 ? sh.fe <= 5 : (sh.fe > 4 && (sh.pz == 32 || sh.pz == 64)) &&
-                                              !(sh.pz == 64 && sh.py * (sh.M / fw) < 100)));
+                                              !((sh.pz == 64 || sh.fe == 6) && sh.py * (sh.M / fw) < 100)));
   if (ctx->z_lanes == -2 || (ctx->z_lanes == 0 && ctx->z_wz == 0 && four_auto)) {
     if (ctx->z_lanes == -2 && !four_ok)
       return fail(ctx, DDS_ERR_UNSUPPORTED, "z pass: the three-stage kernel needs pz 128 or 256 and <= 6 fields "
