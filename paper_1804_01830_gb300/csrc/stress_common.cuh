@@ -79,14 +79,15 @@ __device__ __forceinline__ uint2 ld_cs(const uint2 *p) {
   asm volatile("ld.global.cs.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
   return v;
 }
-__device__ __forceinline__ unsigned ld_cs(const unsigned *p) {
+// Cached in L1: values whose neighbours in the same sector a later load takes.
+__device__ __forceinline__ unsigned ld_ca(const unsigned *p) {
   unsigned v;
-  asm volatile("ld.global.cs.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
-__device__ __forceinline__ uint16_t ld_cs(const uint16_t *p) {
+__device__ __forceinline__ uint16_t ld_ca(const uint16_t *p) {
   uint16_t v;
-  asm volatile("ld.global.cs.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  asm volatile("ld.global.ca.u16 %0, [%1];" : "=h"(v) : "l"(p));
   return v;
 }
 

@@ -246,16 +246,19 @@ __device__ __forceinline__ float2 r2c_post(float2 a, float2 c, float2 wk, float 
   return make_float2(scale * (E.x + (wk.x * O.x - wk.y * O.y)), scale * (E.y + (wk.x * O.y + wk.y * O.x)));
 }
 
-// Complex pair (x[2n], x[2n+1]) of one density line (zero beyond nx).
+// Complex pair (x[2n], x[2n+1]) of one density line (zero beyond nx).  BF16 pairs are two or
+// four bytes of a 32-byte sector, whose rest other loads of the warp take: they are cached
+// in L1 (as streaming loads, an evaluation of 181x128x64, 18 families, 482 against 470 us,
+// 250x64x32, six families, 145 against 132).
 template <bool BF16>
 __device__ __forceinline__ float2 load_pair(const void *rho, long o, int n2x, int nx, bool even) {
   if (BF16) {
     const uint16_t *r = (const uint16_t *)rho;
     if (even) {                                 // both values in one aligned 32-bit word
-      const uint32_t w = ld_cs(reinterpret_cast<const unsigned *>(r + o));
+      const uint32_t w = ld_ca(reinterpret_cast<const unsigned *>(r + o));
       return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
     }
-    return make_float2(bf16_to_f32(ld_cs(r + o)), n2x + 1 < nx ? bf16_to_f32(ld_cs(r + o + 1)) : 0.f);
+    return make_float2(bf16_to_f32(ld_ca(r + o)), n2x + 1 < nx ? bf16_to_f32(ld_ca(r + o + 1)) : 0.f);
   }
   const float *r = (const float *)rho;
   if (even) return ld_cs(reinterpret_cast<const float2 *>(r + o));
@@ -341,7 +344,8 @@ k_x_fwd_reg(Shape sh, Collapse col, GroupList gl, const void *__restrict__ rho_v
   if (live) {
     // one family at a time, all its loads in flight: two cost registers that the later stages
     // lack (GaN layer 0.197 -> 0.194 ms, 256x256x64 in BF16 0.104 -> 0.088 ms), except for short
-    // BF16 rows read value by value (101x90x77: 0.058 against 0.062 ms)
+    // BF16 rows, whose loads are small (one family at a time: 101x90x77 0.062 against 0.058 ms,
+    // 101x128x64 0.067 against 0.060, 64x128x64, read in quads, 0.0228 against 0.0214)
     constexpr int UNROLL = BF16 && !WIDE && M <= 128 ? 2 : 1;
 #pragma unroll UNROLL
     for (int f = 0; f < nfam; ++f) {
