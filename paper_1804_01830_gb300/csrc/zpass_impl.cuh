@@ -268,11 +268,12 @@ template <int E> struct GRaw<__half, E> {
 // than one more CTA allows (padded z 64, FP16 spectra, four fields: 158, three CTAs): at four
 // CTAs and 128 registers, without spills, 100x100x32 185 -> 161 us an evaluation, 256x128x32
 // 362 -> 298; two fields, FP32, at five CTAs 110 -> 98 and 203 -> 189.  The single field on
-// two lanes is faster left alone (256x256x16, FP32: 114 against 117 us).
+// two lanes is left to the compiler (0: no count; 163 registers.  256x256x16, FP32, 114 us,
+// 117 with a stated count of three).
 template <int E, int G, int FE, typename GT> constexpr int zreg_ctas() {
   constexpr bool half = sizeof(GT) == 2;
   if (E == 8) return FE == 1 ? 6 : (FE == 2 ? 5 : (G == 8 && half ? 4 : 3));
-  if (FE == 1) return G == 2 ? 1 : (G == 1 && half ? 5 : 4);
+  if (FE == 1) return G == 2 ? 0 : (G == 1 && half ? 5 : 4);
   return FE == 2 && half ? 3 : 2;
 }
 
