@@ -433,12 +433,13 @@ cudaError_t launch_zreg(const Shape &sh, const float2 *im, const float2 *in, con
   // Started early, its CTAs would share SMs with the y pass's and so keep that pass's split
   // of L1 and shared memory: worth it only where the launch itself is what takes the time
   // (radial disk, 16384 CTAs: 0.56 against 0.52 ms per evaluation; 32x32x8, 33 CTAs: 16.5
-  // against 19 us) and a row of a warp is at least a 128-byte line.  With four or eight lanes
-  // a column several warps share each line through L1 (early against not: 64x64x16, two
-  // fields, 32 against 27 us; 32x32x32, four fields, 42 against 36; two lanes, 64x128x16, 31
-  // against 35)
+  // against 19 us).  With four or eight lanes a column several warps share each 128-byte line
+  // through L1, so only the smallest grids gain (early against not: padded z 32, two fields,
+  // 20x40x16, 132 CTAs, 17 against 21 us, 64x64x16, 260 CTAs, 32 against 27; padded z 64, two
+  // fields, 32x16x32, 66 CTAs, 27 against 29, four fields, 32x32x32, 132 CTAs, 41 against 36;
+  // two lanes, one field, 64x128x16, 35 -> 31)
   const long ctas = (warps + 3) / 4;
-  const bool early = sh.early && G <= 2 && ctas <= 512;
+  const bool early = sh.early && ctas <= (G <= 2 ? 512 : 4608 / (E * G));
   return launch_pass<k_zreg<E, G, FE, GT>, false>(early, (unsigned)ctas, 128, 0, s, sh, im, in, ks, ksc, om, on, tw);
 }
 
