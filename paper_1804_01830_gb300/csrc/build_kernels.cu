@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(128) k_x_lines_d(Tab T, Comps C, const double 
     buf[n * LD + w] = z;
   }
   __syncthreads();
-  fft_tile<M, W, LD, NT, false, false, false>(buf, tw + tw_offset(M), tid);
+  fft_tile<M, W, LD, NT>(buf, tw + tw_offset(M), tid);
   const double2 *tw2 = tw + tw_offset(2 * M);
   for (int e = tid; e < W * (M + 1); e += NT) {
     const int w = e / (M + 1), k = e % (M + 1);
@@ -439,7 +439,7 @@ __global__ void __launch_bounds__(256) k_y_cols_d(Tab T, Comps C, int M, const d
     buf[n * W + w] = v;
   }
   __syncthreads();
-  fft_tile<P, W, W, NT, false, false, false>(buf, tw + tw_offset(P), tid);
+  fft_tile<P, W, W, NT>(buf, tw + tw_offset(P), tid);
   if (!PAIR) {
     double2 *dst = out + ((long)slot * T.nz + k) * P * cols;
     for (int e = tid; e < P * W; e += NT) {
@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(256) k_z_cols_d(int nz, long cols, const doubl
     if (n > 0 && n < P / 2) buf[(P - n) * W + w] = make_double2(-a.x - b.y, a.y - b.x);   // -conj h1 - i conj h2
   }
   __syncthreads();
-  fft_tile<P, W, W, NT, false, false, false>(buf, tw + tw_offset(P), tid);
+  fft_tile<P, W, W, NT>(buf, tw + tw_offset(P), tid);
   for (int e = tid; e < P * 2 * W; e += NT) {
     const int n = e / (2 * W), q = e % (2 * W);
     if (c0 + q >= cols) continue;

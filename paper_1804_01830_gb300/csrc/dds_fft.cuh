@@ -15,7 +15,8 @@
 // buffer suffices.  Forward transforms are unnormalised, exp(-2 pi i nk / P);
 // inverse ones use exp(+2 pi i nk / P), also unnormalised.
 //
-// Two zero-aware variants serve the zero-padded convolution:
+// Two zero-aware variants of the passes with a runtime line count serve the zero-padded
+// convolution:
 //   ZIN : only the first P/2 inputs are non-zero (the first pass skips the rest);
 //   HOUT: only the first P/2 outputs are wanted (the last pass stores only them).
 #pragma once
@@ -162,21 +163,9 @@ __device__ __forceinline__ C tw_load(const C* tw, int idx) {
   return __ldg(tw + idx);
 }
 
-// Address of element n of line w in a tile of W lines.  With PADB > 0 every block
-// of PADB rows is shifted by W elements: the first pass writes rows R0 apart, and
-// without the shift the W-element groups of the butterflies a warp handles at once
-// land on the same shared-memory banks whenever the tile is narrower than 16 lines.
-template <int LD, int PADB, int W>
-__device__ __forceinline__ int tidx(int n, int w) {
-  return n * LD + w + (PADB > 0 ? (n / PADB) * W : 0);
-}
-template <int P, int LD, int PADB, int W>
-__host__ __device__ constexpr int tile_elems() {
-  return P * LD + (PADB > 0 ? (P / PADB) * W : 0);
-}
-
-// One Stockham pass over the tile (see file comment).
-template <int P, int R, int NS, int W, int LD, int PADB, int NT, bool INV, bool ZIN, bool HOUT, typename C>
+// One forward Stockham pass over a tile of W lines, element n of line w at n LD + w (see
+// file comment).
+template <int P, int R, int NS, int W, int LD, int NT, typename C>
 __device__ __forceinline__ void stockham_pass(C* buf, const C* twP, int tid) {
   constexpr int NB = (P / R) * W;
   constexpr int PER = (NB + NT - 1) / NT;
@@ -187,10 +176,7 @@ __device__ __forceinline__ void stockham_pass(C* buf, const C* twP, int tid) {
     if ((NB % NT) == 0 || bi < NB) {
       const int w = bi % W, j = bi / W;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (ZIN && r >= R / 2) v[q][r] = czero<C>();
-        else v[q][r] = buf[tidx<LD, PADB, W>(j + r * (P / R), w)];
-      }
+      for (int r = 0; r < R; ++r) v[q][r] = buf[(j + r * (P / R)) * LD + w];
     }
   }
   __syncthreads();
@@ -204,30 +190,25 @@ __device__ __forceinline__ void stockham_pass(C* buf, const C* twP, int tid) {
 #pragma unroll
         for (int r = 1; r < R; ++r) {
           const C t = tw_load(twP, jm * r * (P / (NS * R)));
-          v[q][r] = cmul_tw<INV>(v[q][r], t);
+          v[q][r] = cmul_tw<false>(v[q][r], t);
         }
       }
-      dft_reg<R, INV>(v[q]);
+      dft_reg<R, false>(v[q]);
       const int base = (j / NS) * NS * R + jm;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (!HOUT || r < R / 2) buf[tidx<LD, PADB, W>(base + r * NS, w)] = v[q][r];
-      }
+      for (int r = 0; r < R; ++r) buf[(base + r * NS) * LD + w] = v[q][r];
     }
   }
   __syncthreads();
 }
 
-// Full length-P FFT of the W lines of a tile.  twP points at the P-table.
-// PADB: 0 for a plain [P][LD] tile, or Plan<P>::r0 for the shifted layout (tidx).
-template <int P, int W, int LD, int NT, bool INV, bool ZIN, bool HOUT, int PADB = 0, typename C>
+// Forward length-P FFT of the W lines of a tile.  twP points at the P-table.
+template <int P, int W, int LD, int NT, typename C>
 __device__ __forceinline__ void fft_tile(C* buf, const C* twP, int tid) {
   using PL = Plan<P>;
-  stockham_pass<P, PL::r0, 1, W, LD, PADB, NT, INV, ZIN, (PL::n == 1) && HOUT>(buf, twP, tid);
-  if constexpr (PL::n >= 2)
-    stockham_pass<P, PL::r1, PL::r0, W, LD, PADB, NT, INV, false, (PL::n == 2) && HOUT>(buf, twP, tid);
-  if constexpr (PL::n >= 3)
-    stockham_pass<P, PL::r2, PL::r0 * PL::r1, W, LD, PADB, NT, INV, false, HOUT>(buf, twP, tid);
+  stockham_pass<P, PL::r0, 1, W, LD, NT>(buf, twP, tid);
+  if constexpr (PL::n >= 2) stockham_pass<P, PL::r1, PL::r0, W, LD, NT>(buf, twP, tid);
+  if constexpr (PL::n >= 3) stockham_pass<P, PL::r2, PL::r0 * PL::r1, W, LD, NT>(buf, twP, tid);
 }
 
 // Variant with a runtime number of interleaved lines L <= LMAX (row pitch L):
