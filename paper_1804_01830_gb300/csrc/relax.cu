@@ -26,11 +26,10 @@ namespace {
 
 struct RelaxCoef {
   int nx, ny, nz;
-  // dt-scaled operator: u_a += sum_b lap[a][b] (u_a[+b] - 2 u_a + u_a[-b])
-  //                          + sum_{b != a} mix[a][b] (4-point cross of u_b in a, b)
-  float lap[3][3];
-  float mix[3][3];
-  float2 lap2[3][3], mix2[3][3];   // the same twice, for packed pairs of cells
+  // dt-scaled operator: u_a += sum_b lap2[a][b] (u_a[+b] - 2 u_a + u_a[-b])
+  //                          + sum_{b != a} mix2[a][b] (4-point cross of u_b in a, b),
+  // each value twice, for packed pairs of cells
+  float2 lap2[3][3], mix2[3][3];
   // ghost layers: first derivatives 1/(2 h) and the factors of Eq. 18b
   float inv2h[3];
   float two_dz;      // 2 dz
@@ -421,10 +420,10 @@ RelaxCoef relax_coef(const dds_ctx *ctx, double *dt_out) {
   const double dt = hmin * hmin / (5.0 * A - 3.0 * B);
   for (int a = 0; a < 3; ++a) {
     for (int b = 0; b < 3; ++b) {
-      r.lap[a][b] = (float)(dt * (a == b ? A : B) / (h[b] * h[b]));
-      r.mix[a][b] = a == b ? 0.f : (float)(dt * (A - B) / (4.0 * h[a] * h[b]));
-      r.lap2[a][b] = make_float2(r.lap[a][b], r.lap[a][b]);
-      r.mix2[a][b] = make_float2(r.mix[a][b], r.mix[a][b]);
+      const float lap = (float)(dt * (a == b ? A : B) / (h[b] * h[b]));
+      const float mix = a == b ? 0.f : (float)(dt * (A - B) / (4.0 * h[a] * h[b]));
+      r.lap2[a][b] = make_float2(lap, lap);
+      r.mix2[a][b] = make_float2(mix, mix);
     }
     r.inv2h[a] = (float)(1.0 / (2.0 * h[a]));
   }
