@@ -443,8 +443,8 @@ template <int PX, bool STEP>
 cudaError_t launch_march_px(const RelaxCoef &r, const float *u, const float *in, const float *phi, float *out, bool early,
                             cudaStream_t s) {
   using C = March<PX>;
-  // Layers per chunk: 16, or 8 or 4 where that would leave CTA slots (two per SM) idle.
-  // Longer chunks restart the march less often, but leave an emptier last wave (step on
+  // Layers per chunk: 16 where that makes two full waves (two CTAs per SM each), 8 where that
+  // makes one, else 4.  Longer chunks restart the march less often, but leave an emptier last wave (step on
   // 256x256x128: 8 / 16 / 32 / 64 layers 82 / 77 / 82 / 81 us; 512x512x16: 8 / 16 layers
   // 49 / 51 us; 100x90x40: 4 / 8 / 16 layers 9 / 12 / 20 us).
   int dev = 0, sms = 0;
