@@ -444,15 +444,20 @@ cudaError_t launch_march_px(const RelaxCoef &r, const float *u, const float *in,
                             cudaStream_t s) {
   using C = March<PX>;
   // Layers per chunk: 16 where that makes two full waves (two CTAs per SM each), 8 where that
-  // makes one, else 4.  Longer chunks restart the march less often, but leave an emptier last wave (step on
-  // 256x256x128: 8 / 16 / 32 / 64 layers 82 / 77 / 82 / 81 us; 512x512x16: 8 / 16 layers
-  // 49 / 51 us; 100x90x40: 4 / 8 / 16 layers 9 / 12 / 20 us).
+  // makes one, else 4.  Longer chunks restart the march less often, but leave an emptier last
+  // wave (step on 256x256x128: 8 / 16 / 32 / 64 layers 82 / 77 / 82 / 81 us; 512x512x16: 8 /
+  // 16 layers 49 / 51 us; 100x90x40: 4 / 8 / 16 layers 9 / 12 / 20 us).  Shorter still while
+  // all chunks are resident at once: a layer's chain and the two ghost planes are then all the
+  // time (1 / 2 / 4 layers, ten steps and the total: 16x16x4 49 / 62 / 91 us, 64x64x8 47 / 54 /
+  // 65, 64x64x64, 512 CTAs at one layer, 86 / 71 / 84; the total alone, 16x16x4 8.4 / 9.1 / 12.4)
   int dev = 0, sms = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (err != cudaSuccess) return err;
   const long tiles = (long)((r.nx + C::TX - 1) / C::TX) * ((r.ny + C::TY - 1) / C::TY);
-  const int kz = tiles * ((r.nz + 15) / 16) >= 4 * sms ? 16 : (tiles * ((r.nz + 7) / 8) >= 2 * sms ? 8 : 4);
+  auto ctas = [&](int layers) { return tiles * ((r.nz + layers - 1) / layers); };
+  int kz = ctas(16) >= 4 * sms ? 16 : (ctas(8) >= 2 * sms ? 8 : 4);
+  while (kz > 1 && ctas(kz / 2) <= 2 * sms) kz /= 2;
   const dim3 grid((unsigned)((r.nx + C::TX - 1) / C::TX), (unsigned)((r.ny + C::TY - 1) / C::TY),
                   (unsigned)((r.nz + kz - 1) / kz));
   const int vec = r.nx % 4 == 0 && ((uintptr_t)u & 15) == 0;
